@@ -152,6 +152,10 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
   return v;
 }
+// v = the word at a where pred holds (no branch)
+__device__ __forceinline__ void lds_u32_if(uint32_t &v, uint32_t a, bool pred) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.shared.u32 %0, [%1];\n\t}" : "+r"(v) : "r"(a), "r"(static_cast<uint32_t>(pred)));
+}
 __device__ __forceinline__ int4 lds_s32x4(uint32_t a) {
   int4 v;
   asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
