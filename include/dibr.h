@@ -266,8 +266,8 @@ dibr_status dibr_synthesize_batch_static(int n, const dibr_image *imgs, const di
  *   ctas_per_sm    CTAs resident per SM at most;
  *   load_mode      1: one bulk copy per input row; 2/3/4: 3-D tensor boxes whose inner
  *                  rows are 16 / 128 / 256 bytes; 5: 2-D tensor boxes of 256 bytes.
- *                  A mode that does not fit an image's width or alignment falls back to
- *                  mode 5, which fits every image;
+ *                  A mode that does not fit an image's width falls back to mode 5; images
+ *                  whose rows are not 16-byte aligned always take mode 1;
  *   l2_prefetch    1: each CTA prefetches its later input rows into L2 at launch;
  *                  2: it does not;
  *   rows_per_unit  rows per work unit of a batched launch (dibr_synthesize_batch and

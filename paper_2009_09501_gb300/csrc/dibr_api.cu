@@ -200,30 +200,31 @@ dibr_status dibr_ctx::plan_band(int W, int H, int depth_src, const uint8_t *in, 
                                BandArgs &a, int &smem, int &per_sm) {
   a.W = W;
   a.H = H;
-  a.nch = (W + kChunk - 1) / kChunk;
-  a.nc = round_up(a.nch, 32);  // one 16-pixel chunk per consumer thread
+  a.out_mode = out_mode_of(a.outputs, a.out, a.out_pitch);
+  a.nch = chunks_of(W);
+  a.nchz = zchunks_of(W, a.out_mode);
+  a.nc = round_up(a.nchz, 32);  // one 16-pixel chunk per thread
   a.zguard = zguard;
-  // how rows reach shared memory: the tuned mode when the image allows it, else the
-  // automatic choice (one bulk copy per row when rows are whole 16-byte units)
-  const bool aligned = (reinterpret_cast<uintptr_t>(in) & 15u) == 0 && (pitch & 15) == 0;
+  // how rows reach shared memory: one bulk copy per row of the 16-byte units it touches,
+  // unless the tuning asks for tensor boxes and the image allows them
+  const bool aligned = rows_aligned(in, pitch);
+  a.ragged = !aligned || a.out_mode != OM_ALIGNED || maps_ragged(a.outputs, a.out, a.depth_pitch);
   int mode = tuning.load_mode;
   const int row = 3 * W;
   auto fits = [&](int m) {
-    if (m == 1) return aligned && row % 16 == 0;
     if (m == 2) return aligned && row % 16 == 0;
     if (m == 3) return aligned && row % 128 == 0;
     if (m == 4) return aligned && row % 256 == 0;
-    return m == 5;
+    return m == 5 && aligned;
   };
-  if (mode == 0) mode = fits(1) ? 1 : 5;
-  if (!fits(mode)) mode = 5;
+  if (!fits(mode)) mode = mode > 1 && aligned ? 5 : 1;
   a.row_bytes = row;
   a.in = in;
   a.in_pitch = pitch;
   if (mode == 1) {
     a.load_mode = LM_BULK;
-    a.nbox = 1;
-    a.box_bytes = row;
+    a.nbox = 0;
+    a.box_bytes = 0;
     a.box_step = 0;
   } else if (mode <= 4) {
     const int inner = mode == 2 ? 16 : mode == 3 ? 128 : 256;
@@ -240,31 +241,17 @@ dibr_status dibr_ctx::plan_band(int W, int H, int depth_src, const uint8_t *in, 
     a.box_bytes = kBoxBytes;
   }
   a.l2_prefetch = tuning.l2_prefetch == 1 ? 1 : 0;
-  a.srow = round_up(std::max(a.nbox * a.box_bytes, 48 * a.nch), 128);
+  a.srow = std::max(slot_bytes(W, aligned), round_up(a.nbox * a.box_bytes, 128));
   a.depth_src = depth_src;
-  const int min_nb = depth_src == DS_BINOM5 ? 4 : 2;
-  const int max_nb = tuning.ring_slots > 0 ? std::max(min_nb, std::min(kMaxRing, tuning.ring_slots)) : kMaxRing;
-  // at most 128 registers per thread (the kernel's launch bound) and 2048 threads per SM
-  const int max_per = std::max(1, std::min(65536 / (a.nc * 128), 2048 / a.nc));
-  auto per_for = [&](int nb) {
-    const int tot = band_smem_layout(nb, a.srow, a.nch, a.nc / 32, zguard).total;
-    if (tot > max_smem) return 0;
-    int per = std::min(max_per, smem_per_sm / (tot + 1024));
-    if (tuning.ctas_per_sm > 0) per = std::min(per, tuning.ctas_per_sm);
-    return per;
-  };
-  int best = 0;
-  for (int nb = min_nb; nb <= max_nb; ++nb) best = std::max(best, per_for(nb));
-  if (best < 1) {
+  BandPlan plan;
+  const BandLimits lim{max_smem, smem_per_sm, tuning.ring_slots, tuning.ctas_per_sm};
+  if (!plan_smem(plan, lim, a.nc, a.srow, a.nch, a.nchz, zguard, depth_src == DS_BINOM5 ? 4 : 2)) {
     set_error("width %d needs more shared memory than the device offers", W);
     return DIBR_E_INVALID;
   }
-  int nb = min_nb;
-  for (int k = min_nb; k <= max_nb; ++k)
-    if (per_for(k) == best) nb = k;
-  a.nb = nb;
-  smem = band_smem_layout(nb, a.srow, a.nch, a.nc / 32, zguard).total;
-  per_sm = best;
+  a.nb = plan.nb;
+  smem = plan.smem;
+  per_sm = plan.per;
   a.grid = std::max(1, std::min(H, num_sms * per_sm));
   a.row0 = 0;
   a.row1 = H;
@@ -275,12 +262,12 @@ dibr_status dibr_ctx::plan_band(int W, int H, int depth_src, const uint8_t *in, 
 }
 
 dibr_status dibr_ctx::encode_input(BandArgs &a, const uint8_t *dev_rgb, int64_t pitch) {
+  if (a.load_mode == LM_BULK) return DIBR_OK;  // no tensor map needed
   auto enc = get_encoder();
   if (!enc) {
     set_error("cuTensorMapEncodeTiled is unavailable");
     return DIBR_E_CUDA;
   }
-  if (a.load_mode == LM_BULK) return DIBR_OK;  // no tensor map needed
   CUresult r;
   if (a.load_mode == LM_T3) {
     const cuuint64_t inner = static_cast<cuuint64_t>(a.tinner);
@@ -307,24 +294,11 @@ dibr_status dibr_ctx::encode_input(BandArgs &a, const uint8_t *dev_rgb, int64_t 
   return DIBR_OK;
 }
 
-// Every requested RGB output and the output pitch are 16-byte aligned: whole 16-column
-// chunks are stored as three 16-byte words.
-static int aligned_rgb_outputs(const BandArgs &a) {
-  uintptr_t bits = static_cast<uintptr_t>(a.out_pitch);
-  for (int i = 0; i < O_COUNT; ++i)
-    if (!is_map_output(i) && (a.outputs & kOutBits[i])) bits |= reinterpret_cast<uintptr_t>(a.out[i]);
-  return (bits & 15u) == 0 ? 1 : 0;
-}
-
-static bool tma_ok(const uint8_t *p, int64_t pitch) {
-  return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (pitch & 15) == 0;
-}
-
 // Enqueues the whole pipeline for one image whose input and outputs are in device memory.
 dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p, const dibr_outputs *o) {
   const int W = img->width, H = img->height;
   const uint8_t *in = img->rgb;
-  int64_t pitch = img->pitch;
+  const int64_t pitch = img->pitch;
   // this launch may overlap the previous one (see below) only if that was the last work
   // on a stream the context owns
   const bool may_overlap = owns_stream && prev_band;
@@ -337,29 +311,13 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   };
   auto meets = [](const Span &x, const Span &y) { return x.lo < y.hi && y.lo < x.hi; };
   bool scratch = false;  // context buffers written before the band kernel
-  bool realigned = false;
-  if (!tma_ok(in, pitch)) {
-    scratch = true;
-    realigned = true;
-    // TMA needs a 16-byte aligned base and pitch: repack into an aligned device buffer
-    const int64_t ap = round_up(3 * W, 16);
-    dibr_status s = ensure(realign, static_cast<size_t>(ap) * H);
-    if (s != DIBR_OK) return s;
-    cudaError_t e = cudaMemcpy2DAsync(realign.ptr, ap, in, pitch, 3 * static_cast<size_t>(W), H,
-                                      cudaMemcpyDeviceToDevice, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "repacking the input");
-    in = realign.ptr;
-    pitch = ap;
-  }
   int depth_src = p->depth_rule == DIBR_DEPTH_LUMA_BINOM5 ? DS_BINOM5
                   : p->depth_rule == DIBR_DEPTH_LUMA     ? DS_LUMA
                                                          : DS_GLOBAL;
   BandArgs &a = args;
   int smem = 0, per_sm = 1;
   const int zguard = band_tables(p);
-  dibr_status s = plan_band(W, H, depth_src, in, pitch, zguard, a, smem, per_sm);
-  if (s != DIBR_OK) return s;
-  if ((s = encode_input(a, in, pitch)) != DIBR_OK) return s;
+  dibr_status s;
   Span cur_depth;  // the cross-bilateral depth this frame's band launch reads
   if (depth_src == DS_GLOBAL) {
     scratch = true;  // the band launch waits for the cross-bilateral one
@@ -373,7 +331,7 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     xbf_half ^= 1;
     cur_depth = span(dd, dp, H, W);
     const Span xin = span(in, pitch, H, 3 * static_cast<int64_t>(W));
-    bool after = may_overlap && !realigned && !meets(cur_depth, prev_in) && !meets(cur_depth, prev_depth);
+    bool after = may_overlap && !meets(cur_depth, prev_in) && !meets(cur_depth, prev_depth);
     for (int i = 0; i < O_COUNT; ++i)
       if (prev_out[i].hi && (meets(xin, prev_out[i]) || meets(cur_depth, prev_out[i]))) after = false;
     cudaError_t e = launch_xbf(in, pitch, W, H, p->xbf_radius, p->xbf_sigma_s, p->xbf_sigma_r, dd, dp, stream,
@@ -401,26 +359,34 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     const uint32_t maps = DIBR_OUT_DEPTH | DIBR_OUT_HOLES;
     const int64_t vp = (p->outputs & rgb) ? o->pitch : round_up(3 * W, 16);
     const int64_t hp = (p->outputs & maps) ? o->depth_pitch : round_up(W, 16);
+    // scratch views start as far from a 16-byte boundary as the caller's outputs, so that all
+    // rows of the launch are aligned alike
+    uintptr_t lead = 0;
+    for (int i = 0; i < O_COUNT; ++i)
+      if (p->outputs & rgb & kOutBits[i]) lead = reinterpret_cast<uintptr_t>(a.out[i]) & 15u;
+    const size_t view_bytes = (static_cast<size_t>(vp) * H + 16 + 15) / 16 * 16;
+    const size_t holes_bytes = (static_cast<size_t>(hp) * H + 15) / 16 * 16;
     size_t need = 0;
-    if (!(p->outputs & DIBR_OUT_LEFT)) need += static_cast<size_t>(vp) * H;
-    if (!(p->outputs & DIBR_OUT_RIGHT)) need += static_cast<size_t>(vp) * H;
-    if (!(p->outputs & DIBR_OUT_HOLES)) need += static_cast<size_t>(hp) * H;
+    if (!(p->outputs & DIBR_OUT_LEFT)) need += view_bytes;
+    if (!(p->outputs & DIBR_OUT_RIGHT)) need += view_bytes;
+    if (!(p->outputs & DIBR_OUT_HOLES)) need += holes_bytes;
     if (need && (s = ensure(inpaint_scratch, 2 * need)) != DIBR_OK) return s;
     size_t off = inpaint_half * need;
     inpaint_half ^= 1;
-    auto take = [&](int slot, uint32_t bit, int64_t rows_pitch) {
+    auto take = [&](int slot, uint32_t bit, size_t bytes, size_t at) {
       if (p->outputs & bit) return;
-      a.out[slot] = inpaint_scratch.ptr + off;
-      off += static_cast<size_t>(rows_pitch) * H;
+      a.out[slot] = inpaint_scratch.ptr + off + at;
+      off += bytes;
     };
-    take(O_LEFT, DIBR_OUT_LEFT, vp);
-    take(O_RIGHT, DIBR_OUT_RIGHT, vp);
-    take(O_HOLES, DIBR_OUT_HOLES, hp);
+    take(O_LEFT, DIBR_OUT_LEFT, view_bytes, lead);
+    take(O_RIGHT, DIBR_OUT_RIGHT, view_bytes, lead);
+    take(O_HOLES, DIBR_OUT_HOLES, holes_bytes, 0);
     a.out_pitch = vp;
     a.depth_pitch = hp;
     a.outputs |= DIBR_OUT_LEFT | DIBR_OUT_RIGHT | DIBR_OUT_HOLES;
   }
-  a.fast_store = aligned_rgb_outputs(a);
+  if ((s = plan_band(W, H, depth_src, in, pitch, zguard, a, smem, per_sm)) != DIBR_OK) return s;
+  if ((s = encode_input(a, in, pitch)) != DIBR_OK) return s;
   // Overlap with the previous band launch on the stream when neither reads or writes what
   // the other writes: this launch then starts in the SMs the previous one leaves and only
   // its exit waits for it.
@@ -449,7 +415,7 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     if (cudaPeekAtLastError() == cudaErrorNotReady) cudaGetLastError();  // (not an error)
     a.grid = std::max(1, std::min(a.grid, (num_sms * per_sm + fif - 1) / fif));
   }
-  cudaError_t e = launch_band(a, smem, per_sm, stream);
+  cudaError_t e = launch_band(a, smem, stream);
   a.overlap = 0;
   a.grid = full_grid;
   if (e != cudaSuccess) return cuda_fail(e, "band kernel launch");
@@ -715,8 +681,6 @@ dibr_status dibr_ctx::synthesize_banded(const dibr_image *img, const dibr_params
   int smem = 0, per_sm = 1;
   const int depth_src = p->depth_rule == DIBR_DEPTH_LUMA_BINOM5 ? DS_BINOM5 : DS_LUMA;
   const int zguard = band_tables(p);
-  if ((s = plan_band(W, H, depth_src, stage_in.ptr, ap, zguard, a, smem, per_sm)) != DIBR_OK) return s;
-  if ((s = encode_input(a, stage_in.ptr, ap)) != DIBR_OK) return s;
   a.depth_in = nullptr;
   a.depth_in_pitch = 0;
   for (int i = 0; i < O_COUNT; ++i) a.out[i] = (p->outputs & kOutBits[i]) ? stage_out.ptr + offs[i] : nullptr;
@@ -724,7 +688,8 @@ dibr_status dibr_ctx::synthesize_banded(const dibr_image *img, const dibr_params
   a.depth_pitch = dp;
   a.outputs = p->outputs;
   a.warp_mode = p->warp_mode;
-  a.fast_store = aligned_rgb_outputs(a);
+  if ((s = plan_band(W, H, depth_src, stage_in.ptr, ap, zguard, a, smem, per_sm)) != DIBR_OK) return s;
+  if ((s = encode_input(a, stage_in.ptr, ap)) != DIBR_OK) return s;
   const int slots = a.grid;  // CTAs of a whole-frame launch
   auto band_row = [&](int k) { return static_cast<int>(static_cast<int64_t>(k) * H / bands); };
   // the copy streams start after the work already queued on the context's stream
@@ -748,7 +713,7 @@ dibr_status dibr_ctx::synthesize_banded(const dibr_image *img, const dibr_params
     a.row0 = y0;
     a.row1 = y1;
     a.grid = std::max(1, std::min(y1 - y0, slots));
-    e = launch_band(a, smem, per_sm, stream);
+    e = launch_band(a, smem, stream);
     if (e == cudaSuccess) e = cudaEventRecord(ev_comp[k], stream);
     if (e != cudaSuccess) return cuda_fail(e, "band kernel launch");
     ++launches;
@@ -844,7 +809,7 @@ dibr_status dibr_ctx::synthesize_staged(const dibr_image *img, const dibr_params
 
 void dibr_ctx::release_buffers() {
   release_band_pipeline();
-  for (DevBuf *b : {&stage_in, &stage_out, &realign, &xbf_depth, &inpaint_scratch, &inpaint_order}) {
+  for (DevBuf *b : {&stage_in, &stage_out, &xbf_depth, &inpaint_scratch, &inpaint_order}) {
     dev_free(b->ptr);
     b->ptr = nullptr;
     b->bytes = 0;

@@ -34,9 +34,18 @@
 // wait that gives up sets a bit of the status word and the CTA unwinds after letting its
 // own copies land.
 //
+// Rows may start anywhere (tight rows of a width that is no multiple of 16, an offset base): a
+// ring slot then holds the 16-byte units a row touches, its first byte at `lead`; the luminance
+// shifts the words it loads, B's colour loads start there.  Output rows are met halfway: the
+// z-buffer keeps target x at x + shift, with the row's shift (0..15) chosen so that every thread's
+// 16 targets start on a 16-byte boundary of the output row; only the two chunks cut by the row's
+// ends are stored by words and bytes.  That is the RAG template flag: a 4031 x 3023 photo with
+// tight rows 780 -> 107 us, 1366 x 768 side by side 29.6 -> 10.0 us (repacked by a strided copy
+// and stored by bytes before); aligned images keep instances without it.
+//
 // Instances: the requested outputs are read from the arguments, or fixed at compile time for
 // the two sets the workloads use (left + right + anaglyph, anaglyph alone; binomial depth,
-// forward warp, 16-byte aligned rows), which drops the output branches and the state they
+// forward warp), which drops the output branches and the state they
 // keep live.  The fixed-set instances in bands of kTmemMinRows rows or more keep the vertical
 // cascade's 32 words per thread in tensor memory between one row's A and the next, so that B
 // and C have those registers.
@@ -123,25 +132,71 @@ __device__ __forceinline__ void luma_row(const uint32_t (&b)[NB], uint32_t (&y)[
   for (int j = 0; j < N; j += 2) mul_luma(y[j], y[j + 1]);
 }
 
+// Words of a row in shared memory from byte s + off on (s < 16: where the row's first byte
+// sits in its slot, the same for every thread of a row; off a multiple of 8): 16-byte loads of
+// the units that hold them, then a shift by whole words (one of four cases, the same for the
+// whole warp) and one funnel shift per word.
+template <int N>
+__device__ __forceinline__ void lds_ragged(uint32_t row, uint32_t s, int off, uint32_t (&w)[N]) {
+  constexpr int kUnits = (4 * N + 15 + 15) / 16;
+  const uint32_t a = row + s + static_cast<uint32_t>(off);
+  uint32_t l[4 * kUnits + 1];
+#pragma unroll
+  for (int i = 0; i < kUnits; ++i) {
+    const uint4 u = lds_u32x4((a & ~15u) + 16u * i);
+    l[4 * i] = u.x; l[4 * i + 1] = u.y; l[4 * i + 2] = u.z; l[4 * i + 3] = u.w;
+  }
+  l[4 * kUnits] = 0u;
+  const uint32_t sh = (a & 3u) * 8u;
+  switch ((a >> 2) & 3u) {
+    case 0:
+#pragma unroll
+      for (int i = 0; i < N; ++i) w[i] = __funnelshift_r(l[i], l[i + 1], sh);
+      break;
+    case 1:
+#pragma unroll
+      for (int i = 0; i < N; ++i) w[i] = __funnelshift_r(l[i + 1], l[i + 2], sh);
+      break;
+    case 2:
+#pragma unroll
+      for (int i = 0; i < N; ++i) w[i] = __funnelshift_r(l[i + 2], l[i + 3], sh);
+      break;
+    default:
+#pragma unroll
+      for (int i = 0; i < N; ++i) w[i] = __funnelshift_r(l[i + 3], l[i + 4], sh);
+      break;
+  }
+}
+
 // Luminance of columns x0-2 .. x0+17 (clamped to [0, W-1]) of one input row held in
-// shared memory, as 10 words of two 16-bit lanes: yp[2q] = columns (4q, 4q+2) and
-// yp[2q+1] = (4q+1, 4q+3) of the window, the layout the vertical cascade works on.
-__device__ __forceinline__ void luma20(const uint8_t *row, int x0, int W, uint32_t (&yp)[10]) {
-  // bytes 3*x0-8 .. 3*x0+55 (8-byte and 16-byte aligned loads); column j of the window at
-  // byte 2+3j.  At the row's ends the loads reach past it into neighbouring shared memory
-  // (another ring slot, the summaries before the ring, the depth row after it); those
-  // columns are replaced below by the row's first or last column.
+// shared memory from byte s of `row` on, as 10 words of two 16-bit lanes: yp[2q] = columns
+// (4q, 4q+2) and yp[2q+1] = (4q+1, 4q+3) of the window, the layout the vertical cascade
+// works on.  RAG: any s < 16; otherwise s = 0.
+template <bool RAG>
+__device__ __forceinline__ void luma20(const uint8_t *row, uint32_t s, int x0, int W, uint32_t (&yp)[10]) {
+  // bytes 3*x0-8 .. 3*x0+55 of the row; column j of the window at byte 2+3j.  At the row's
+  // ends the loads reach past it into neighbouring shared memory (another ring slot, the
+  // summaries before the ring, the depth row after it); those columns are replaced below by
+  // the row's first or last column.
   uint32_t b[17];
-  const uint2 l = *reinterpret_cast<const uint2 *>(row + 3 * x0 - 8);
-  const uint4 m0 = *reinterpret_cast<const uint4 *>(row + 3 * x0);
-  const uint4 m1 = *reinterpret_cast<const uint4 *>(row + 3 * x0 + 16);
-  const uint4 m2 = *reinterpret_cast<const uint4 *>(row + 3 * x0 + 32);
-  const uint2 r = *reinterpret_cast<const uint2 *>(row + 3 * x0 + 48);
-  b[0] = l.x; b[1] = l.y;
-  b[2] = m0.x; b[3] = m0.y; b[4] = m0.z; b[5] = m0.w;
-  b[6] = m1.x; b[7] = m1.y; b[8] = m1.z; b[9] = m1.w;
-  b[10] = m2.x; b[11] = m2.y; b[12] = m2.z; b[13] = m2.w;
-  b[14] = r.x; b[15] = r.y; b[16] = r.y;
+  if (RAG) {
+    uint32_t w[16];
+    lds_ragged<16>(smem_addr(row), s, 3 * x0 - 8, w);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) b[i] = w[i];
+    b[16] = w[15];
+  } else {
+    const uint2 l = *reinterpret_cast<const uint2 *>(row + 3 * x0 - 8);
+    const uint4 m0 = *reinterpret_cast<const uint4 *>(row + 3 * x0);
+    const uint4 m1 = *reinterpret_cast<const uint4 *>(row + 3 * x0 + 16);
+    const uint4 m2 = *reinterpret_cast<const uint4 *>(row + 3 * x0 + 32);
+    const uint2 r = *reinterpret_cast<const uint2 *>(row + 3 * x0 + 48);
+    b[0] = l.x; b[1] = l.y;
+    b[2] = m0.x; b[3] = m0.y; b[4] = m0.z; b[5] = m0.w;
+    b[6] = m1.x; b[7] = m1.y; b[8] = m1.z; b[9] = m1.w;
+    b[10] = m2.x; b[11] = m2.y; b[12] = m2.z; b[13] = m2.w;
+    b[14] = r.x; b[15] = r.y; b[16] = r.y;
+  }
   uint32_t y[20];
   luma_row<20, 2>(b, y);
 #pragma unroll
@@ -162,7 +217,7 @@ __device__ __forceinline__ void luma20(const uint8_t *row, int x0, int W, uint32
       yp[8] = (yp[8] & 0xFFFFu) | yl;
       yp[9] = (yp[9] & 0xFFFFu) | yl;
     } else if (x0 + 18 > W) {
-      const uint8_t *pl = row + 3 * (W - 1);
+      const uint8_t *pl = row + s + 3 * (W - 1);
       const uint32_t ylast = luma8(pl[0], pl[1], pl[2]);
 #pragma unroll
       for (int j = 3; j < 20; ++j) {
@@ -175,11 +230,22 @@ __device__ __forceinline__ void luma20(const uint8_t *row, int x0, int W, uint32
 
 // Luminance of the 16 columns x0 .. x0+15 of a row in shared memory, packed 4 per word
 // (columns past the row's end take whatever their bytes give: they are never used).
-__device__ __forceinline__ uint4 luma16(const uint8_t *row, int x0) {
-  const uint4 m0 = *reinterpret_cast<const uint4 *>(row + 3 * x0);
-  const uint4 m1 = *reinterpret_cast<const uint4 *>(row + 3 * x0 + 16);
-  const uint4 m2 = *reinterpret_cast<const uint4 *>(row + 3 * x0 + 32);
-  const uint32_t b[13] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w, m2.x, m2.y, m2.z, m2.w, m2.w};
+template <bool RAG>
+__device__ __forceinline__ uint4 luma16(const uint8_t *row, uint32_t s, int x0) {
+  uint32_t b[13];
+  if (RAG) {
+    uint32_t w[12];
+    lds_ragged<12>(smem_addr(row), s, 3 * x0, w);
+#pragma unroll
+    for (int i = 0; i < 12; ++i) b[i] = w[i];
+  } else {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const uint4 m = *reinterpret_cast<const uint4 *>(row + 3 * x0 + 16 * q);
+      b[4 * q] = m.x; b[4 * q + 1] = m.y; b[4 * q + 2] = m.z; b[4 * q + 3] = m.w;
+    }
+  }
+  b[12] = b[11];
   uint32_t y[16];
   luma_row<16, 0>(b, y);
   uint32_t d[4];
@@ -289,34 +355,59 @@ __device__ __forceinline__ uint32_t avg_up(uint32_t a, uint32_t b) {
   return (a | b) - (((a ^ b) >> 1) & 0x7F7F7F7Fu);
 }
 
+// Bytes b0 .. b1 - 1 of the words w at p.
 template <int N>
-__device__ __forceinline__ void store_bytes(uint8_t *p, const uint32_t (&w)[N], int nbytes) {
+__device__ __forceinline__ void store_bytes(uint8_t *p, const uint32_t (&w)[N], int b0, int b1) {
 #pragma unroll
   for (int b = 0; b < 4 * N; ++b)
-    if (b < nbytes) p[b] = static_cast<uint8_t>(bsel(w, b));
+    if (b >= b0 && b < b1) p[b] = static_cast<uint8_t>(bsel(w, b));
 }
 
-// 16 packed colours (48 bytes) at p: three 16-byte stores when the chunk is whole and
-// the row 16-byte aligned (`fast`), else byte stores of the npx pixels.
-__device__ __forceinline__ void store48(uint8_t *p, const uint32_t (&w)[12], int npx, bool fast) {
-  if (fast) {
-    uint4 *q = reinterpret_cast<uint4 *>(p);
-    q[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    q[1] = make_uint4(w[4], w[5], w[6], w[7]);
-    q[2] = make_uint4(w[8], w[9], w[10], w[11]);
-  } else {
-    store_bytes(p, w, 3 * npx);
+// 16 packed colours (48 bytes) at p, 16-byte aligned.
+__device__ __forceinline__ void store48(uint8_t *p, const uint32_t (&w)[12]) {
+  uint4 *q = reinterpret_cast<uint4 *>(p);
+  q[0] = make_uint4(w[0], w[1], w[2], w[3]);
+  q[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  q[2] = make_uint4(w[8], w[9], w[10], w[11]);
+}
+
+// The chunks of the warp that the row's ends cut (thread t's chunk holds the row's bytes
+// 48 t - 3 c .. + 47 as 12 words, 4-byte aligned): one word per lane, so that the whole warp
+// shares the stores of its one or two cut chunks.
+__device__ __forceinline__ void store_edge(uint8_t *row, const uint32_t (&w)[12], int t, int c, int W) {
+  const int lane = t & 31, last = (W + c) >> 4;
+#pragma unroll 1
+  for (int e = 0; e < 2; ++e) {
+    const int te = e == 0 ? 0 : last;  // (the chunk: the same for the whole warp)
+    if (e == 0 ? c == 0 : (((W + c) & 15) == 0 || (c > 0 && last == 0))) continue;
+    if ((te & ~31) != (t & ~31)) continue;
+    uint32_t mine = 0u;
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      const uint32_t u = __shfl_sync(kAll, w[i], te & 31);
+      if (lane == i) mine = u;
+    }
+    const int b0 = 48 * te - 3 * c + 4 * lane;
+    if (lane < 12) {
+      if (b0 >= 0 && b0 + 4 <= 3 * W) {
+        *reinterpret_cast<uint32_t *>(row + b0) = mine;
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (b0 + q >= 0 && b0 + q < 3 * W) row[b0 + q] = static_cast<uint8_t>(mine >> (8 * q));
+      }
+    }
   }
 }
 
-__device__ __forceinline__ void store24(uint8_t *p, const uint32_t (&w)[6], int npx) {
-  if (npx == 8 && (reinterpret_cast<uintptr_t>(p) & 7u) == 0) {
+__device__ __forceinline__ void store24(uint8_t *p, const uint32_t (&w)[6], int b0, int b1) {
+  if (b0 == 0 && b1 == 24 && (reinterpret_cast<uintptr_t>(p) & 7u) == 0) {
     uint2 *q = reinterpret_cast<uint2 *>(p);
     q[0] = make_uint2(w[0], w[1]);
     q[1] = make_uint2(w[2], w[3]);
     q[2] = make_uint2(w[4], w[5]);
   } else {
-    store_bytes(p, w, 3 * npx);
+    store_bytes(p, w, b0, b1);
   }
 }
 
@@ -325,7 +416,7 @@ __device__ __forceinline__ void store16(uint8_t *p, uint4 v, int npx) {
     *reinterpret_cast<uint4 *>(p) = v;
   } else {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    store_bytes(p, w, npx);
+    store_bytes(p, w, 0, npx);
   }
 }
 
@@ -414,28 +505,49 @@ struct Job {
   const CUtensorMap *tmap;  // tensor-box load modes only
   const uint8_t *depth_in;
   int64_t depth_in_pitch;
+  const int32_t *lut_n;     // Fig. 3 gather: 510 * s_L(d)
   uint8_t *out[O_COUNT];
   int64_t out_pitch, depth_pitch;
-  int W, H, nch, row_bytes, load_mode, nbox, box_bytes, box_step;
+  int W, H, nch, nchz, row_bytes, load_mode, nbox, box_bytes, box_step;
   uint32_t outputs;
-  int l2_prefetch, fast_store;
+  int l2_prefetch, out_mode;
+
+  // where row r's first byte sits in its ring slot (rows that are not whole 16-byte units)
+  __device__ __forceinline__ uint32_t lead(int r) const {
+    return static_cast<uint32_t>(reinterpret_cast<uintptr_t>(in) + static_cast<uintptr_t>(r) * in_pitch) & 15u;
+  }
+  // Columns the targets of row y, view v are moved by, so that every 16-column chunk of an
+  // output row starts on a 16-byte boundary (chunk t then holds columns 16 t - shift ..):
+  // 3 * shift = the row's address modulo 16, and 3 * 11 = 1 modulo 16.  The side-by-side
+  // frame alone: 24-byte half chunks on 8-byte boundaries, 3 * 3 = 1 modulo 8, each view by
+  // its own half's address.
+  __device__ __forceinline__ int shift(int y, int v) const {
+    if (out_mode == OM_SHIFT) {
+      const uint8_t *const p = outputs & DIBR_OUT_ANAGLYPH ? out[O_ANA] : outputs & DIBR_OUT_LEFT ? out[O_LEFT] : out[O_RIGHT];
+      return static_cast<int>(11u * static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p) + static_cast<uintptr_t>(y) * out_pitch)) & 15;
+    }
+    if (out_mode == OM_HALF) {
+      const uintptr_t p = reinterpret_cast<uintptr_t>(out[O_HSBS]) + static_cast<uintptr_t>(y) * out_pitch;
+      return 2 * (static_cast<int>(3u * static_cast<uint32_t>(p + (v ? 3 * (W / 2) : 0))) & 7);
+    }
+    return 0;
+  }
 };
 
 // Shared-memory regions of one CTA.
 struct Shm {
   uint64_t *full;   // ring-slot mbarriers
-  uint64_t *bdone;  // [2] every warp has scattered the row (B)
+  uint64_t *bdone;  // [2] every warp has written the row's targets (B)
   uint64_t *sdone;  // [2] every warp has published its summary and cleared its targets (C)
-  uint2 *lut;       // per 255 - depth: byte offsets of the left / right targets
-  int32_t *lut_n;   // Fig. 3 gather: 510 * s_L(d) (in the z-buffer region)
+  uint2 *lut;       // per 255 - depth: byte offsets of the left / right targets (gather: shifts)
   uint8_t *wsum;    // [parity][view][warp] uint4 {has, first entry, last entry, 0}
   uint8_t *ring, *drow;
   uint32_t zb;      // shared address of the z-buffer region
   int nb, srow, zlen, zstride, zguard;
 };
 
-__device__ __forceinline__ Shm carve(uint8_t *smem, int nb, int srow, int nch, int nwarps, int zguard) {
-  const BandSmem L = band_smem_layout(nb, srow, nch, nwarps, zguard);
+__device__ __forceinline__ Shm carve(uint8_t *smem, int nb, int srow, int nch, int nchz, int nwarps, int zguard) {
+  const BandSmem L = band_smem_layout(nb, srow, nch, nchz, nwarps, zguard);
   Shm m;
   m.full = reinterpret_cast<uint64_t *>(smem + L.bar);
   m.bdone = reinterpret_cast<uint64_t *>(smem + L.flags + 8);
@@ -445,27 +557,24 @@ __device__ __forceinline__ Shm carve(uint8_t *smem, int nb, int srow, int nch, i
   m.ring = smem + L.ring;
   m.drow = smem + L.drow;
   m.zb = smem_addr(smem + L.zb);
-  m.lut_n = reinterpret_cast<int32_t *>(smem + L.zb);
   m.nb = nb;
   m.srow = srow;
-  m.zlen = nch * kChunk;
+  m.zlen = nchz * kChunk;
   m.zstride = L.zstride;
   m.zguard = zguard;
   return m;
 }
 
-// Shift tables into shared memory (all threads; a barrier must follow).  lut[255 - d] =
-// {4 * (-hL[d]), 4 * (-hR[d])}: a source at column x with depth d lands on target x - h.
+// Shift tables into shared memory (all threads; a barrier must follow).  Forward warp:
+// lut[255 - d] = {4 * (-hL[d]), 4 * (-hR[d])}: a source at column x with depth d lands on
+// target x - h.  Gather: lut[255 - d] = {hL[d], hR[d]}: target x samples column x + h.
 template <bool FWD>
-__device__ __forceinline__ void fill_luts(const Shm &m, const int32_t *lut_h, const int32_t *lut_n) {
+__device__ __forceinline__ void fill_luts(const Shm &m, const int32_t *lut_h) {
   for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-    if (FWD) {
-      const int32_t h = lut_h[255 - i];
-      const int nl = -static_cast<int16_t>(h & 0xFFFF), nr = -(h >> 16);  // |h| <= 512
-      m.lut[i] = make_uint2(static_cast<uint32_t>(4 * nl), static_cast<uint32_t>(4 * nr));
-    } else {
-      m.lut_n[i] = lut_n[i];
-    }
+    const int32_t h = lut_h[255 - i];
+    const int hl = static_cast<int16_t>(h & 0xFFFF), hr = h >> 16;  // |h| <= 512
+    m.lut[i] = FWD ? make_uint2(static_cast<uint32_t>(-4 * hl), static_cast<uint32_t>(-4 * hr))
+                   : make_uint2(static_cast<uint32_t>(hl), static_cast<uint32_t>(hr));
   }
 }
 
@@ -486,12 +595,11 @@ __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, unsign
 // processed before (each per-row mbarrier completes one phase per row); both are advanced
 // here.  Returns false when a bounded wait gave up (the status word is set and the copies
 // in flight have landed).
-// OUTS: the requested outputs when fixed at compile time (the stereo set, every output row
-// 16-byte aligned: whole chunks stored as 16-byte words), 0 when read from the arguments.
-//
+// OUTS: the requested outputs when fixed at compile time, 0 when read from the arguments.
+// RAG: input or output rows may start anywhere; otherwise all start on 16-byte boundaries.
 // TM: the vertical cascade's 32 words wait in tensor memory (at tmem, this thread's lane)
 // between one row's A and the next, so that B and C have those registers.
-template <int DS, bool FWD, uint32_t OUTS = 0, bool TM = false>
+template <int DS, bool FWD, uint32_t OUTS, bool RAG, bool TM>
 __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int ye, uint32_t &kbase,
                                          uint32_t &nrows, int *status,
                                          unsigned long long timeout_ns, uint32_t tmem = 0u) {
@@ -514,6 +622,7 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
   int issued = 0;
   const int lw = 32 * (nwarps >> 1);  // first thread of the loading warp
   const bool loader = __shfl_sync(kAll, (tid >> 5) == (nwarps >> 1), 0);
+  const bool end_units = RAG || (a.row_bytes & 15) != 0;  // some row's units reach past its bytes
   auto issue_loads = [&](int upto) {
     upto = min(upto, nload);
     if (tid == lw && issued == 0 && a.load_mode != LM_BULK) prefetch_tensormap(a.tmap);
@@ -522,10 +631,40 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
       const int s = static_cast<int>(g - ring_div(g) * nb);
       uint8_t *dst = m.ring + s * m.srow;
       if (a.load_mode == LM_BULK) {
+        // a row is the 16-byte units its bytes touch: one bulk copy of those that lie inside
+        // the image, and the few bytes at the image's very ends (units shared with other
+        // memory) by plain loads, so that nothing outside the image is read
+        if (!end_units) {
+          if (tid == lw) {
+            mbar_arrive_expect_tx(&m.full[s], static_cast<uint32_t>(a.row_bytes));
+            bulk_load(dst, a.in + static_cast<int64_t>(la + k) * a.in_pitch, static_cast<uint32_t>(a.row_bytes),
+                      &m.full[s]);
+          }
+          continue;
+        }
+        const int r = la + k;
+        const uintptr_t p = reinterpret_cast<uintptr_t>(a.in) + static_cast<uintptr_t>(r) * a.in_pitch;
+        const uint32_t ld = RAG ? static_cast<uint32_t>(p) & 15u : 0u;
+        uint32_t lo = 0u, hi = (ld + static_cast<uint32_t>(a.row_bytes) + 15u) & ~15u;  // bytes from unit ld of the slot
+        if (end_units && (r == 0 || r + 1 == H || a.in_pitch < 16)) {
+          const uintptr_t base = reinterpret_cast<uintptr_t>(a.in), first = p - ld;
+          const uintptr_t last = base + static_cast<uintptr_t>(H - 1) * a.in_pitch + a.row_bytes;
+          if (first < base) lo = 16u;
+          if (first + hi > last) hi -= 16u;
+          if (hi < lo) hi = lo;
+          const uint32_t end = ld + static_cast<uint32_t>(a.row_bytes);
+          for (uint32_t q = ld + lane; q < min(lo, end); q += 32) dst[q] = reinterpret_cast<const uint8_t *>(first)[q];
+          for (uint32_t q = max(hi, ld) + lane; q < end; q += 32) dst[q] = reinterpret_cast<const uint8_t *>(first)[q];
+          fence_proxy_async_smem();
+          __syncwarp();
+        }
         if (tid == lw) {
-          mbar_arrive_expect_tx(&m.full[s], static_cast<uint32_t>(a.row_bytes));
-          bulk_load(dst, a.in + static_cast<int64_t>(la + k) * a.in_pitch, static_cast<uint32_t>(a.row_bytes),
-                    &m.full[s]);
+          if (hi > lo) {
+            mbar_arrive_expect_tx(&m.full[s], hi - lo);
+            bulk_load(dst + lo, reinterpret_cast<const uint8_t *>(p - ld + lo), hi - lo, &m.full[s]);
+          } else {
+            mbar_arrive(&m.full[s]);
+          }
         }
       } else {
         if (tid == lw) mbar_arrive_expect_tx(&m.full[s], static_cast<uint32_t>(a.nbox * a.box_bytes));
@@ -545,8 +684,11 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
     // optionally, the band's later rows go to L2 now
     if (a.l2_prefetch) {
       if (a.load_mode == LM_BULK) {
-        for (int k = nb + lane; k < nload; k += 32)
-          bulk_prefetch_l2(a.in + static_cast<int64_t>(la + k) * a.in_pitch, static_cast<uint32_t>(a.row_bytes));
+        for (int k = nb + lane; k < nload; k += 32) {
+          const uintptr_t p = reinterpret_cast<uintptr_t>(a.in) + static_cast<uintptr_t>(la + k) * a.in_pitch;
+          const uintptr_t lo = (p + 15) & ~static_cast<uintptr_t>(15), hi = (p + a.row_bytes) & ~static_cast<uintptr_t>(15);
+          if (hi > lo) bulk_prefetch_l2(reinterpret_cast<const uint8_t *>(lo), static_cast<uint32_t>(hi - lo));
+        }
       } else {
         for (int j = lane; j < (nload - nb) * a.nbox; j += 32) {
           const int k = nb + j / a.nbox, i = j % a.nbox;
@@ -564,8 +706,6 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
   // the warp's 32 chunks are all whole (every warp of a row but possibly the last):
   // warp-uniform fast paths for its depth row, clears and stores
   const bool wfull = __all_sync(kAll, npx == kChunk);
-  const bool fast_store = OUTS ? true : a.fast_store != 0;
-  const bool wfast = wfull && fast_store;
   const int x0c = min(x0, (a.nch - 1) * kChunk);  // clamped: loads stay inside the buffers
   const int warp_lo = (tid & ~31) * kChunk;
   const int warp_hi = min(W, warp_lo + 32 * kChunk);
@@ -606,7 +746,7 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
       const int r = min(max(ys + i, 0), H - 1);
       if (r >= la && r < lb && (i == -2 || r != min(max(ys + i - 1, 0), H - 1))) wait_row(r);
       uint32_t yq[10], hq[8], V[8];
-      luma20(slot(r), x0c, W, yq);
+      luma20<RAG>(slot(r), RAG ? a.lead(r) : 0u, x0c, W, yq);
       binom_h(yq, hq);
       vc.feed(hq, V);
     }
@@ -630,8 +770,13 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
   auto par = [&](int y) { return (rix(y) >> 1) & 1u; };
   auto arrive_b = [&](int y) { mbar_arrive(bbar(y)); };
 
-  // ---- A: the depth of row y (registers, 4 per word), 255 - depth into the depth row
-  auto phase_a = [&](int y) -> uint4 {
+  // depth output rows that are not 16-byte aligned are written by B, a byte per lane
+  auto depth_bytes = [&](int y) {
+    return RAG && want_depth && ((reinterpret_cast<uintptr_t>(a.out[O_DEPTH]) + static_cast<uintptr_t>(y) * a.depth_pitch) & 15u) != 0;
+  };
+
+  // ---- A: the depth of row y (4 columns per word), 255 - depth into the depth row
+  auto phase_a = [&](int y) {
     uint4 d;
     if (binom) {
       const int r2 = y + 2;
@@ -641,7 +786,7 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
       uint32_t V[8];
       if (r2 < H) {
         uint32_t yq[10], hq[8];
-        luma20(slot(r2), x0c, W, yq);
+        luma20<RAG>(slot(r2), RAG ? a.lead(r2) : 0u, x0c, W, yq);
         binom_h(yq, hq);
         if (TM) {
           tmem_load_wait32(t);
@@ -662,7 +807,7 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
       d = round_depth(V);
     } else if (DS == DS_LUMA) {
       wait_row(y);
-      d = luma16(slot(y), x0c);
+      d = luma16<RAG>(slot(y), RAG ? a.lead(y) : 0u, x0c);
     } else {
       wait_row(y);  // B reads the row's colours
       d = make_uint4(0u, 0u, 0u, 0u);
@@ -677,29 +822,77 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
         }
       }
     }
-    if (want_depth && active) store16(a.out[O_DEPTH] + static_cast<int64_t>(y) * a.depth_pitch + x0, d, npx);
-    if (FWD && (wfull || own_chunk)) *reinterpret_cast<uint4 *>(m.drow + x0) = make_uint4(~d.x, ~d.y, ~d.z, ~d.w);
-    return d;
+    if (want_depth && active && !depth_bytes(y)) store16(a.out[O_DEPTH] + static_cast<int64_t>(y) * a.depth_pitch + x0, d, npx);
+    if (wfull || own_chunk) *reinterpret_cast<uint4 *>(m.drow + x0) = make_uint4(~d.x, ~d.y, ~d.z, ~d.w);
   };
 
-  // ---- B: the forward warp of row y: the warp's 512 sources, consecutive lanes on
-  // consecutive columns, so that the atomics of one instruction land on distinct banks
-  // (shifts vary slowly); all shared loads of four steps are issued before their atomics
+  // ---- B: the targets of row y from the warp's 512 columns, consecutive lanes on consecutive
+  // columns, so that the shared accesses of one instruction fall on distinct banks (shifts
+  // vary slowly); all shared loads of four steps are issued before their atomics
   auto phase_b = [&](int y) {
-    if (!FWD) return;
-    // every warp has cleared its targets of row y - 2, the previous user of this z-buffer
-    // (the band's first two rows use the buffers cleared before the band)
+    // every warp has cleared (gather: read) its targets of row y - 2, the previous user of this
+    // z-buffer (the band's first two rows use the buffers cleared before the band)
     if (y >= ys + 2 && !warp_wait(m.sdone + (rix(y - 2) & 1u), par(y - 2), timeout_ns)) timed_out = true;
     const int xb = warp_lo + lane;
-    const uint32_t ob = 3u * static_cast<uint32_t>(xb);
-    const uint32_t cws = smem_addr(slot(y)) + (ob & ~3u);  // the lane's colours: +96 bytes per step
+    const uint32_t rs = smem_addr(slot(y)), lead = RAG ? a.lead(y) : 0u;
+    const uint32_t ob = 3u * static_cast<uint32_t>(xb) + lead;
+    const uint32_t cws = rs + (ob & ~3u);  // the lane's colours: +96 bytes per step
     const uint32_t sh = (ob & 3u) * 8u;
-    const uint32_t ds = smem_addr(m.drow) + static_cast<uint32_t>(xb);
+    const uint32_t dr = smem_addr(m.drow), ds = dr + static_cast<uint32_t>(xb);
     const uint32_t ls = smem_addr(m.lut);
     const int p = y & 1;
-    const uint32_t bl = zrow(p, 0) + 4u * static_cast<uint32_t>(xb);
-    const uint32_t br = zrow(p, 1) + 4u * static_cast<uint32_t>(xb);
-    if (warp_hi - warp_lo == 32 * kChunk) {
+    const uint32_t bl = zrow(p, 0) + 4u * static_cast<uint32_t>(xb + (RAG ? a.shift(y, 0) : 0));
+    const uint32_t br = zrow(p, 1) + 4u * static_cast<uint32_t>(xb + (RAG ? a.shift(y, 1) : 0));
+    const bool dbytes = OUTS ? false : depth_bytes(y);
+    uint8_t *const dp = dbytes ? a.out[O_DEPTH] + static_cast<int64_t>(y) * a.depth_pitch : nullptr;
+    if (!FWD) {
+      // Fig. 3 literally: target x samples column trunc(x + s(d)) = x + floor(s(d)), but 0
+      // when -1 < x + s(d) < 0; its own column when that lies outside the row.  From the row
+      // in shared memory into the z-buffers, from which C formats it like a row of the forward
+      // warp without holes (1080p: 8.8 us with byte loads from global memory in C, 7.8 so).
+      const int ng = (warp_hi - warp_lo + 127) >> 7;  // groups of 4 x 32 columns holding some
+#pragma unroll 1
+      for (int g = 0; g < ng; ++g) {
+        uint32_t f[4];
+        int sx[2][4];
+        bool out = false;  // some sample lies outside the row
+#pragma unroll
+        for (int j = 0; j < 4; ++j) f[j] = lds_u8(dr + min(xb + 32 * (4 * g + j), warp_hi - 1));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int x = min(xb + 32 * (4 * g + j), warp_hi - 1);
+          const uint2 h = lds_u32x2(ls + 8u * f[j]);
+          sx[0][j] = x + static_cast<int>(h.x);
+          sx[1][j] = x + static_cast<int>(h.y);
+          out |= static_cast<unsigned>(sx[0][j]) >= static_cast<unsigned>(W) || static_cast<unsigned>(sx[1][j]) >= static_cast<unsigned>(W);
+        }
+        if (__any_sync(kAll, out)) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+              if (static_cast<unsigned>(sx[v][j]) >= static_cast<unsigned>(W))
+                sx[v][j] = sx[v][j] == -1 && a.lut_n[255u - f[j]] % 510 != 0 ? 0 : min(xb + 32 * (4 * g + j), warp_hi - 1);
+        }
+        uint32_t c[2][4];
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t o = rs + lead + 3u * static_cast<uint32_t>(sx[v][j]);
+            c[v][j] = __funnelshift_r(lds_u32(o & ~3u), lds_u32((o & ~3u) + 4u), (o & 3u) * 8u);
+          }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int x = xb + 32 * (4 * g + j);
+          if (x < warp_hi) {
+            sts_u32(bl + 512u * g + 128u * j, c[0][j]);
+            sts_u32(br + 512u * g + 128u * j, c[1][j]);
+            if (dbytes) dp[x] = static_cast<uint8_t>(255u - f[j]);
+          }
+        }
+      }
+    } else if (warp_hi - warp_lo == 32 * kChunk && !dbytes) {
       scatter4<0>(ds, cws, sh, ls, bl, br);
       scatter4<1>(ds, cws, sh, ls, bl, br);
       scatter4<2>(ds, cws, sh, ls, bl, br);
@@ -707,7 +900,6 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
     } else {
       // the row's last, partial warp: columns from warp_hi on do not exist (their loads
       // read column warp_hi - 1, so that they stay in the row; their atomics are skipped)
-      const uint32_t rs = smem_addr(slot(y)), dr = smem_addr(m.drow);
       const int ng = (warp_hi - warp_lo + 127) >> 7;  // groups of 4 x 32 columns holding some
 #pragma unroll 1
       for (int g = 0; g < ng; ++g) {
@@ -715,7 +907,7 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const uint32_t xc = static_cast<uint32_t>(min(xb + 32 * (4 * g + j), warp_hi - 1));
-          const uint32_t ca = rs + ((3u * xc) & ~3u);
+          const uint32_t ca = rs + ((3u * xc + lead) & ~3u);
           fv[j] = lds_u8(dr + xc);
           cw[2 * j] = lds_u32(ca);
           cw[2 * j + 1] = lds_u32(ca + 4);
@@ -725,11 +917,12 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
         for (int j = 0; j < 4; ++j) lt[j] = lds_u32x2(ls + 8u * fv[j]);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const bool in = xb + 32 * (4 * g + j) < warp_hi;
+          const int x = xb + 32 * (4 * g + j);
           const uint32_t e = __byte_perm(__funnelshift_r(cw[2 * j], cw[2 * j + 1], sh), fv[j], 0x4210);
           const uint32_t off = 512u * static_cast<uint32_t>(g) + 128u * j;
-          reds_min_at_if<0>(bl + off + lt[j].x, e, in);
-          reds_min_at_if<0>(br + off + lt[j].y, e, in);
+          reds_min_at_if<0>(bl + off + lt[j].x, e, x < warp_hi);
+          reds_min_at_if<0>(br + off + lt[j].y, e, x < warp_hi);
+          if (dbytes && x < warp_hi) dp[x] = static_cast<uint8_t>(255u - fv[j]);
         }
       }
     }
@@ -740,61 +933,32 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
 
   // this lane's clears: 16 bytes at warp_lo + 4 * lane + 128 q targets, q = 0..3
   const uint32_t clr_off = 4u * static_cast<uint32_t>(warp_lo + 4 * lane);
-  auto phase_c = [&](int y, uint4 d) {
-    // every warp has scattered row y: its targets are final and its ring slot is free
+  const int zt = min(tid, a.nchz - 1) * kChunk;  // the thread's first target (clamped)
+  const bool clear_all = warp_lo + 32 * kChunk <= m.zlen;
+  auto phase_c = [&](int y) {
+    // every warp has written row y's targets: they are final and its ring slot is free
     if (!warp_wait(bbar(y), par(y), timeout_ns)) timed_out = true;
     if (loader) issue_loads((y - la) + 1 + nb);
-    const uint8_t *grow = a.in + static_cast<int64_t>(y) * a.in_pitch;
     const int p = y & 1;
-    // Formatting and stores of one view's 16 targets: the view itself, its half of the
-    // side-by-side frame and, after the right view, the anaglyph (red from the left view,
-    // green and blue from the right: in the packed words, the bytes at offsets 0 mod 3).
-    const int64_t ro = static_cast<int64_t>(y) * a.out_pitch;
-    const bool fast = wfast || (fast_store && npx == kChunk);
-    uint32_t wl[12];
-    auto emit_view = [&](int v, const uint32_t (&kv)[16]) {
-      if (!wfull && !active) return;
-      uint32_t w[12];
-      pack16(kv, w);
-      if (v == 0) {
-        if (want_l) store48(a.out[O_LEFT] + ro + 3 * x0, w, npx, fast);
+    // the columns of the thread's targets: tx[v] + j, of which lo[v] <= j < hi[v] lie in the row
+    // (thread t's targets are the columns 16 t .. 16 t + 15 less the row's shift)
+    int sv[2], tx[2], lo[2], hi[2];
 #pragma unroll
-        for (int i = 0; i < 12; ++i) wl[i] = w[i];
-      } else {
-        if (want_r) store48(a.out[O_RIGHT] + ro + 3 * x0, w, npx, fast);
-        if (want_ana) {
-          uint32_t wa[12];
-#pragma unroll
-          for (int i = 0; i < 12; ++i) {
-            const uint32_t M = i % 3 == 0 ? 0xFF0000FFu : i % 3 == 1 ? 0x00FF0000u : 0x0000FF00u;
-            wa[i] = (wl[i] & M) | (w[i] & ~M);
-          }
-          store48(a.out[O_ANA] + ro + 3 * x0, wa, npx, fast);
-        }
-      }
-      if (want_hsbs) {
-        uint32_t c8[8], h6[6];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) c8[j] = avg_up(kv[2 * j], kv[2 * j + 1]);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          h6[3 * q] = __byte_perm(c8[4 * q], c8[4 * q + 1], 0x4210);
-          h6[3 * q + 1] = __byte_perm(c8[4 * q + 1], c8[4 * q + 2], 0x5421);
-          h6[3 * q + 2] = __byte_perm(c8[4 * q + 2], c8[4 * q + 3], 0x6542);
-        }
-        // W is even, so chunks hold whole pairs; the left view fills the left half
-        store24(a.out[O_HSBS] + ro + 3 * ((v == 0 ? 0 : W / 2) + x0 / 2), h6, npx / 2);
-      }
-    };
+    for (int v = 0; v < 2; ++v) {
+      sv[v] = !RAG ? 0 : v == 0 || a.out_mode == OM_HALF ? a.shift(y, v) : sv[0];
+      tx[v] = x0 - sv[v];
+      lo[v] = RAG ? min(max(-tx[v], 0), kChunk) : 0;
+      hi[v] = RAG ? min(max(W - tx[v], 0), kChunk) : npx;
+    }
     uint32_t k[2][16];
     uint32_t hole[2] = {0u, 0u};
     if (FWD) {
-      const uint32_t rowmask = npx >= kChunk ? 0xFFFFu : ((1u << npx) - 1u);
       uint32_t mm[2], fe[2], cl[2], cr[2], lanes[2];
 
 #pragma unroll
       for (int v = 0; v < 2; ++v) {
-        const uint32_t za = zrow(p, v) + 4u * static_cast<uint32_t>(x0c);
+        const uint32_t rowmask = (hi[v] >= kChunk ? 0xFFFFu : ((1u << hi[v]) - 1u)) & (RAG ? ~((1u << lo[v]) - 1u) : kAll);
+        const uint32_t za = zrow(p, v) + 4u * static_cast<uint32_t>(zt);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const uint4 u = lds_u32x4(za + 16u * q);
@@ -818,6 +982,11 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
         sts_u32x4(wsum_at(p, v, warp), make_uint4(ln != 0u ? 1u : 0u, wf, wl, 0u));  // (same value, every lane)
         mm[v] = mk;
         lanes[v] = ln;
+        if (RAG && lo[v] > 0) {  // targets left of the row: empty for the sweep
+#pragma unroll
+          for (int j = 0; j < 15; ++j)
+            if (j < lo[v]) k[v][j] = kEmpty;
+        }
       }
       // this warp's targets are read: clear them for row y + 2 (consecutive lanes on
       // consecutive 16-byte words: no bank conflicts), then tell the other warps that its
@@ -825,7 +994,7 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
       __syncwarp();
       const uint4 e4 = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
       const uint32_t c0 = zrow(p, 0) + clr_off, c1 = zrow(p, 1) + clr_off;
-      if (wfull) {
+      if (clear_all) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           sts_u32x4(c0 + 512u * q, e4);
@@ -845,12 +1014,12 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
       // filled entry, from the summaries -- only where a warp below (above) exists: the
       // holes at the row's ends need nothing from the other warps
       bool need = false;
-      const bool below_exists = warp_lo > 0, above_exists = warp_hi < W;
 #pragma unroll
       for (int v = 0; v < 2; ++v) {
+        const bool below_exists = warp_lo > 0, above_exists = warp_lo + 32 * kChunk < W + sv[v];
         const uint32_t lower = lanes[v] & ltm, upper = lanes[v] & gtm;
-        need |= active && ((below_exists && lower == 0u && !(mm[v] & 1u)) ||
-                           (above_exists && upper == 0u && !((mm[v] >> ((npx - 1) & 15)) & 1u)));
+        need |= hi[v] > lo[v] && ((below_exists && lower == 0u && !(mm[v] & 1u)) ||
+                                  (above_exists && upper == 0u && !((mm[v] >> ((hi[v] - 1) & 15)) & 1u)));
       }
       uint32_t wle[2] = {0u, 0u}, wre[2] = {0u, 0u};
       bool wlh[2] = {false, false}, wrh[2] = {false, false};
@@ -887,69 +1056,139 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
         const uint32_t lower = lanes[v] & ltm, upper = lanes[v] & gtm, mk = mm[v];
         rin[v] = upper ? cr[v] : wre[v];
         lin[v] = lower ? cl[v] : (wlh[v] ? wle[v] : (mk ? fe[v] : rin[v]));
-        hole[v] = ~mk & rowmask;
+        hole[v] = ~mk & 0xFFFFu;
       }
       carry_right2(k[0], k[1], lin[0], lin[1]);
       carry_left_farther2(k[0], k[1], mm[0], mm[1], rin[0], rin[1]);
       // a view of a row without any filled target shows the input row (warp-uniform)
       const bool none0 = lanes[0] == 0u && !wlh[0] && !wrh[0], none1 = lanes[1] == 0u && !wlh[1] && !wrh[1];
       if (none0 || none1) {
+        const uint8_t *grow = a.in + static_cast<int64_t>(y) * a.in_pitch;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          const uint32_t c = active ? rgb_at_global(grow, min(x0 + j, W - 1)) : 0u;
-          if (none0) k[0][j] = c;
-          if (none1) k[1][j] = c;
+          if (none0) k[0][j] = rgb_at_global(grow, min(max(tx[0] + j, 0), W - 1));
+          if (none1) k[1][j] = rgb_at_global(grow, min(max(tx[1] + j, 0), W - 1));
         }
       }
-      emit_view(0, k[0]);
-      emit_view(1, k[1]);
     } else {
-      // Fig. 3 literally: sample trunc(x + s(d)); out of range -> own column
-      mbar_arrive(sbar(y));
-      const uint32_t dw[4] = {d.x, d.y, d.z, d.w};
 #pragma unroll
-      for (int i = 0; i < kChunk; ++i) {
-        const int x = min(x0 + i, W - 1);
-        const int n = m.lut_n[bsel(dw, i)];
-        int sl = (510 * x + n) / 510, sr = (510 * x - n) / 510;
-        if (static_cast<unsigned>(sl) >= static_cast<unsigned>(W)) sl = x;
-        if (static_cast<unsigned>(sr) >= static_cast<unsigned>(W)) sr = x;
-        k[0][i] = active ? rgb_at_global(grow, sl) : 0u;
-        k[1][i] = active ? rgb_at_global(grow, sr) : 0u;
+      for (int v = 0; v < 2; ++v) {
+        const uint32_t za = zrow(p, v) + 4u * static_cast<uint32_t>(zt);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint4 u = lds_u32x4(za + 16u * q);
+          k[v][4 * q] = u.x; k[v][4 * q + 1] = u.y; k[v][4 * q + 2] = u.z; k[v][4 * q + 3] = u.w;
+        }
       }
-      emit_view(0, k[0]);
-      emit_view(1, k[1]);
+      mbar_arrive(sbar(y));
     }
-    if (active && want_holes) {
+    // ---- formats and stores.  The side-by-side frame: each view's pairs into its half (W and
+    // the row's shift are even, so chunks hold whole pairs).
+    const int64_t ro = static_cast<int64_t>(y) * a.out_pitch;
+    if (want_hsbs) {
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        uint32_t c8[8], h6[6];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) c8[j] = avg_up(k[v][2 * j], k[v][2 * j + 1]);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          h6[3 * q] = __byte_perm(c8[4 * q], c8[4 * q + 1], 0x4210);
+          h6[3 * q + 1] = __byte_perm(c8[4 * q + 1], c8[4 * q + 2], 0x5421);
+          h6[3 * q + 2] = __byte_perm(c8[4 * q + 2], c8[4 * q + 3], 0x6542);
+        }
+        store24(a.out[O_HSBS] + ro + 3 * ((v == 0 ? 0 : W / 2) + tx[v] / 2), h6, 3 * (lo[v] / 2), 3 * (hi[v] / 2));
+      }
+    }
+    // The views and the anaglyph (red from the left view, green and blue from the right: in the
+    // packed words, the bytes at offsets 0 mod 3), which share one shift.  Whole chunks go out as
+    // 16-byte words; a warp with a chunk that a row end cuts stores that one word by word.  The
+    // common case is kept free of branches between the views (with them, 4K frames took 33.8
+    // instead of 31.2 us: nothing of one view's stores could be scheduled among the other's
+    // packing).
+    if (want_l || want_r || want_ana) {
+      uint32_t wl[12], wr[12];
+      pack16(k[0], wl);
+      pack16(k[1], wr);
+      auto mix = [&]() {
+#pragma unroll
+        for (int i = 0; i < 12; ++i) {
+          const uint32_t M = i % 3 == 0 ? 0xFF0000FFu : i % 3 == 1 ? 0x00FF0000u : 0x0000FF00u;
+          wl[i] = (wl[i] & M) | (wr[i] & ~M);
+        }
+      };
+      const int64_t o = ro + 3 * static_cast<int64_t>(tx[0]);
+      const bool cut = (sv[0] > 0 && warp == 0) || (((W + sv[0]) & (kChunk - 1)) != 0 && (W + sv[0]) >> 9 == warp);
+      if ((OUTS && !RAG) || a.out_mode != OM_BYTES) {
+        if (!cut) {
+          if (wfull || hi[0] > 0) {  // (every chunk of the warp lies in the row or past its end)
+            if (want_l) store48(a.out[O_LEFT] + o, wl);
+            if (want_r) store48(a.out[O_RIGHT] + o, wr);
+            if (want_ana) {
+              mix();
+              store48(a.out[O_ANA] + o, wl);
+            }
+          }
+        } else {
+          auto store_cut = [&](uint8_t *out, const uint32_t (&w)[12]) {
+            if (lo[0] == 0 && hi[0] == kChunk) store48(out + o, w);
+            store_edge(out + ro, w, tid, sv[0], W);
+          };
+          if (want_l) store_cut(a.out[O_LEFT], wl);
+          if (want_r) store_cut(a.out[O_RIGHT], wr);
+          if (want_ana) {
+            mix();
+            store_cut(a.out[O_ANA], wl);
+          }
+        }
+      } else {
+        if (want_l) store_bytes(a.out[O_LEFT] + o, wl, 3 * lo[0], 3 * hi[0]);
+        if (want_r) store_bytes(a.out[O_RIGHT] + o, wr, 3 * lo[0], 3 * hi[0]);
+        if (want_ana) {
+          mix();
+          store_bytes(a.out[O_ANA] + o, wl, 3 * lo[0], 3 * hi[0]);
+        }
+      }
+    }
+    if (want_holes) {
       // one byte per target: bit 0 a hole of the left view, bit 1 of the right view
-      auto spread4 = [](uint32_t x) { return ((x & 0xFu) * 0x00204081u) & 0x01010101u; };
-      uint4 hv;
-      hv.x = spread4(hole[0]) | (spread4(hole[1]) << 1);
-      hv.y = spread4(hole[0] >> 4) | (spread4(hole[1] >> 4) << 1);
-      hv.z = spread4(hole[0] >> 8) | (spread4(hole[1] >> 8) << 1);
-      hv.w = spread4(hole[0] >> 12) | (spread4(hole[1] >> 12) << 1);
-      store16(a.out[O_HOLES] + static_cast<int64_t>(y) * a.depth_pitch + x0, hv, npx);
+      uint8_t *row = a.out[O_HOLES] + static_cast<int64_t>(y) * a.depth_pitch;
+      if (!RAG || ((reinterpret_cast<uintptr_t>(row) + tx[0]) & 15u) == 0) {
+        auto spread4 = [](uint32_t x) { return ((x & 0xFu) * 0x00204081u) & 0x01010101u; };
+        uint32_t hv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) hv[q] = spread4(hole[0] >> (4 * q)) | (spread4(hole[1] >> (4 * q)) << 1);
+        uint8_t *q = row + tx[0];
+        if (lo[0] == 0 && hi[0] == kChunk) *reinterpret_cast<uint4 *>(q) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
+        else if (hi[0] > lo[0]) store_bytes(q, hv, lo[0], hi[0]);
+      } else {
+        // a row that is not 16-byte aligned: a byte per lane, consecutive lanes on consecutive
+        // targets (step s: target 32 s + lane of the warp, of lane 2 s + lane / 16)
+        const uint32_t both = hole[0] | (hole[1] << 16);
+#pragma unroll 4
+        for (int s = 0; s < 16; ++s) {
+          const uint32_t h = __shfl_sync(kAll, both, 2 * s + (lane >> 4)) >> (lane & 15);
+          const int x = warp_lo - sv[0] + 32 * s + lane;
+          if (x >= 0 && x < W) row[x] = static_cast<uint8_t>((h & 1u) | ((h >> 15) & 2u));
+        }
+      }
     }
   };
 
-  uint4 dcur = make_uint4(0u, 0u, 0u, 0u);
   if (!aborted) {
-    dcur = phase_a(ys);
+    phase_a(ys);
     phase_b(ys);
     arrive_b(ys);
   }
   for (int y = ys; y < ye && !aborted && !timed_out; ++y) {
     // the loader refills the slot of row y as soon as every warp has scattered it
     if (loader && __any_sync(kAll, mbar_test(bbar(y), par(y)))) issue_loads((y - la) + 1 + nb);
-    const bool more = y + 1 < ye;
-    uint4 dnext = make_uint4(0u, 0u, 0u, 0u);
-    if (more) {
-      dnext = phase_a(y + 1);
+    if (y + 1 < ye) {
+      phase_a(y + 1);
       phase_b(y + 1);
       arrive_b(y + 1);
     }
-    phase_c(y, dcur);
-    dcur = dnext;
+    phase_c(y);
   }
 
   // every thread agrees whether the band completed
@@ -985,15 +1224,15 @@ __device__ __forceinline__ void init_barriers(const Shm &m, int nb) {
 // One image: CTA b owns the rows row0 + [b*n/grid, (b+1)*n/grid), n = row1 - row0.
 // TM (fixed-set instances with the binomial depth, bands of kTmemMinRows rows or more): the
 // cascade waits in tensor memory between rows.
-template <int DS, bool FWD, uint32_t OUTS, bool TM>
+template <int DS, bool FWD, uint32_t OUTS, bool RAG, bool TM>
 __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_constant__ BandArgs a) {
   static_assert(!TM || (OUTS != 0 && DS == DS_BINOM5), "tensor memory only in the fixed-set binomial instances");
   // The next launch on the stream may start its set-up while this one runs (programmatic
   // dependent launch); it waits below for this one to complete before any global access.
   griddep_launch_dependents();
   extern __shared__ __align__(128) uint8_t smem[];
-  const Shm m = carve(smem, a.nb, a.srow, a.nch, blockDim.x >> 5, a.zguard);
-  fill_luts<FWD>(m, a.lut_h, a.lut_n);
+  const Shm m = carve(smem, a.nb, a.srow, a.nch, a.nchz, blockDim.x >> 5, a.zguard);
+  fill_luts<FWD>(m, a.lut_h);
   init_barriers(m, a.nb);
   __syncthreads();
   // the work before this launch on the stream (whose results may be this launch's inputs,
@@ -1011,13 +1250,14 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_con
     j.tmap = &a.tmap;
     j.depth_in = a.depth_in;
     j.depth_in_pitch = a.depth_in_pitch;
+    j.lut_n = a.lut_n;
 #pragma unroll
     for (int i = 0; i < O_COUNT; ++i) j.out[i] = a.out[i];
     j.out_pitch = a.out_pitch;
     j.depth_pitch = a.depth_pitch;
-    j.W = a.W; j.H = a.H; j.nch = a.nch; j.row_bytes = a.row_bytes; j.load_mode = a.load_mode;
+    j.W = a.W; j.H = a.H; j.nch = a.nch; j.nchz = a.nchz; j.row_bytes = a.row_bytes; j.load_mode = a.load_mode;
     j.nbox = a.nbox; j.box_bytes = a.box_bytes; j.box_step = a.box_step;
-    j.outputs = a.outputs; j.l2_prefetch = a.l2_prefetch; j.fast_store = a.fast_store;
+    j.outputs = a.outputs; j.l2_prefetch = a.l2_prefetch; j.out_mode = a.out_mode;
     uint32_t kbase = 0, nrows = 0;
     const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     // 32 columns per group of four warps (a warp reaches only its quarter of the lanes),
@@ -1026,7 +1266,7 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_con
     const uint32_t ncols = nwarps <= 4 ? 32u : nwarps <= 8 ? 64u : 128u;
     uint32_t tbase = 0u;
     if (TM) {
-      const uint32_t slot_addr = smem_addr(smem + band_smem_layout(a.nb, a.srow, a.nch, nwarps, a.zguard).flags + 48);
+      const uint32_t slot_addr = smem_addr(smem + band_smem_layout(a.nb, a.srow, a.nch, a.nchz, nwarps, a.zguard).flags + 48);
       if (warp == 0) tmem_alloc(slot_addr, ncols);
       tmem_fence_before_sync();
       __syncthreads();
@@ -1034,7 +1274,7 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_con
       tbase = lds_u32(slot_addr);
     }
     const uint32_t tmem = tbase + ((32u * (warp & 3)) << 16) + 32u * (warp >> 2);
-    run_band<DS, FWD, OUTS, TM>(j, m, ys, ye, kbase, nrows, a.status, a.timeout_ns, tmem);
+    run_band<DS, FWD, OUTS, RAG, TM>(j, m, ys, ye, kbase, nrows, a.status, a.timeout_ns, tmem);
     if (TM) {  // every thread's stores have completed (each store waits for itself)
       tmem_fence_before_sync();
       __syncthreads();
@@ -1048,9 +1288,9 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_con
 // ---------------------------------------------------------------------------------
 // A batch of images in one persistent launch: CTAs pull work units (an image and a
 // range of its rows) from a device counter until none is left.
-// OUTS: every image of the launch has this fixed output set (binomial depth, forward warp,
-// aligned rows); 0: each image's own choices.
-template <uint32_t OUTS>
+// OUTS: every image of the launch has this fixed output set (binomial depth, forward warp);
+// 0: each image's own choices.  RAG: some image's rows are not on 16-byte boundaries.
+template <uint32_t OUTS, bool RAG>
 __global__ void __launch_bounds__(kMaxConsumers, 1) batch_kernel(BatchArgs b) {
   // The next launch of the batch (another group of images, independent of this one) may be
   // placed as soon as every CTA of this one runs: its CTAs take the SM slots this launch
@@ -1059,8 +1299,8 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) batch_kernel(BatchArgs b) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int nwarps = blockDim.x >> 5;
   // the barriers and the unit word sit at the same place in every image's layout
-  const Shm m0 = carve(smem, b.nb, b.srow, b.nch_max, nwarps, b.zguard);
-  const int flags = band_smem_layout(b.nb, b.srow, b.nch_max, nwarps, b.zguard).flags;
+  const Shm m0 = carve(smem, b.nb, b.srow, b.nch_max, b.nchz_max, nwarps, b.zguard);
+  const int flags = band_smem_layout(b.nb, b.srow, b.nch_max, b.nchz_max, nwarps, b.zguard).flags;
   int *unit_s = reinterpret_cast<int *>(smem + flags);
   init_barriers(m0, b.nb);
   // a fixed-set batch keeps each unit's binomial cascade in tensor memory between rows
@@ -1089,35 +1329,35 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) batch_kernel(BatchArgs b) {
     const ImageDesc &dsc = b.descs[un.x];
     // this image's layout (its z-buffer rows as wide as its own row, so that its targets
     // past the row's end are the ones its C clears)
-    const Shm m = carve(smem, b.nb, b.srow, dsc.nch, nwarps, b.zguard);
+    const Shm m = carve(smem, b.nb, b.srow, dsc.nch, dsc.nchz, nwarps, b.zguard);
     Job j;
     j.in = dsc.in;
     j.in_pitch = dsc.in_pitch;
     j.tmap = nullptr;
     j.depth_in = dsc.depth_in;
     j.depth_in_pitch = dsc.depth_in_pitch;
+    j.lut_n = dsc.lut_n;
 #pragma unroll
     for (int i = 0; i < O_COUNT; ++i) j.out[i] = dsc.out[i];
     j.out_pitch = dsc.out_pitch;
     j.depth_pitch = dsc.depth_pitch;
-    j.W = dsc.W; j.H = dsc.H; j.nch = dsc.nch; j.row_bytes = dsc.row_bytes; j.load_mode = LM_BULK;
+    j.W = dsc.W; j.H = dsc.H; j.nch = dsc.nch; j.nchz = dsc.nchz; j.row_bytes = dsc.row_bytes; j.load_mode = LM_BULK;
     j.nbox = 1; j.box_bytes = dsc.row_bytes; j.box_step = 0;
     j.outputs = dsc.outputs; j.l2_prefetch = 0;
-    j.fast_store = ((reinterpret_cast<uintptr_t>(dsc.out[O_ANA]) | reinterpret_cast<uintptr_t>(dsc.out[O_LEFT]) |
-                     reinterpret_cast<uintptr_t>(dsc.out[O_RIGHT]) | static_cast<uintptr_t>(dsc.out_pitch)) & 15u) == 0;
+    j.out_mode = dsc.out_mode;
     const bool fwd = OUTS ? true : dsc.warp_mode == DIBR_WARP_FORWARD;
-    if (fwd) fill_luts<true>(m, dsc.lut_h, dsc.lut_n);
-    else fill_luts<false>(m, dsc.lut_h, dsc.lut_n);
+    if (fwd) fill_luts<true>(m, dsc.lut_h);
+    else fill_luts<false>(m, dsc.lut_h);
     __syncthreads();
     bool ok;
-    if (OUTS) ok = run_band<DS_BINOM5, true, OUTS, TM>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns, tmem);
+    if (OUTS) ok = run_band<DS_BINOM5, true, OUTS, RAG, TM>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns, tmem);
     else switch (dsc.depth_src * 2 + (fwd ? 0 : 1)) {
-      case DS_BINOM5 * 2: ok = run_band<DS_BINOM5, true>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
-      case DS_BINOM5 * 2 + 1: ok = run_band<DS_BINOM5, false>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
-      case DS_LUMA * 2: ok = run_band<DS_LUMA, true>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
-      case DS_LUMA * 2 + 1: ok = run_band<DS_LUMA, false>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
-      case DS_GLOBAL * 2: ok = run_band<DS_GLOBAL, true>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
-      default: ok = run_band<DS_GLOBAL, false>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
+      case DS_BINOM5 * 2: ok = run_band<DS_BINOM5, true, 0, RAG, false>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
+      case DS_BINOM5 * 2 + 1: ok = run_band<DS_BINOM5, false, 0, RAG, false>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
+      case DS_LUMA * 2: ok = run_band<DS_LUMA, true, 0, RAG, false>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
+      case DS_LUMA * 2 + 1: ok = run_band<DS_LUMA, false, 0, RAG, false>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
+      case DS_GLOBAL * 2: ok = run_band<DS_GLOBAL, true, 0, RAG, false>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
+      default: ok = run_band<DS_GLOBAL, false, 0, RAG, false>(j, m, un.y, un.z, kbase, nrows, b.status, b.timeout_ns); break;
     }
     if (!ok) break;
   }
@@ -1146,10 +1386,10 @@ cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
   return e;
 }
 
-template <int DS, bool FWD, uint32_t OUTS = 0, bool TM = false>
+template <int DS, bool FWD, uint32_t OUTS, bool RAG, bool TM>
 cudaError_t launch_band_t(const BandArgs &a, int smem_bytes, cudaStream_t st) {
   static std::atomic<uint64_t> done{0};
-  cudaError_t e = allow_smem(band_kernel<DS, FWD, OUTS, TM>, done);
+  cudaError_t e = allow_smem(band_kernel<DS, FWD, OUTS, RAG, TM>, done);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.grid);
@@ -1161,38 +1401,51 @@ cudaError_t launch_band_t(const BandArgs &a, int smem_bytes, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, band_kernel<DS, FWD, OUTS, TM>, a);
+  e = cudaLaunchKernelEx(&cfg, band_kernel<DS, FWD, OUTS, RAG, TM>, a);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <uint32_t OUTS, bool RAG>
+cudaError_t launch_fixed(const BandArgs &a, int smem_bytes, cudaStream_t st) {
+  // bands of a few rows do not repay a CTA's tensor-memory allocation
+  return a.row1 - a.row0 >= kTmemMinRows * a.grid ? launch_band_t<DS_BINOM5, true, OUTS, RAG, true>(a, smem_bytes, st)
+                                                  : launch_band_t<DS_BINOM5, true, OUTS, RAG, false>(a, smem_bytes, st);
+}
+
+template <bool RAG>
+cudaError_t launch_any(const BandArgs &a, int smem_bytes, cudaStream_t st) {
+  const bool fwd = a.warp_mode == DIBR_WARP_FORWARD;
+  switch (a.depth_src) {
+    case DS_BINOM5:
+      return fwd ? launch_band_t<DS_BINOM5, true, 0, RAG, false>(a, smem_bytes, st)
+                 : launch_band_t<DS_BINOM5, false, 0, RAG, false>(a, smem_bytes, st);
+    case DS_LUMA:
+      return fwd ? launch_band_t<DS_LUMA, true, 0, RAG, false>(a, smem_bytes, st)
+                 : launch_band_t<DS_LUMA, false, 0, RAG, false>(a, smem_bytes, st);
+    default:
+      return fwd ? launch_band_t<DS_GLOBAL, true, 0, RAG, false>(a, smem_bytes, st)
+                 : launch_band_t<DS_GLOBAL, false, 0, RAG, false>(a, smem_bytes, st);
+  }
 }
 
 }  // namespace
 
-cudaError_t launch_band(const BandArgs &a, int smem_bytes, int ctas_per_sm, cudaStream_t st) {
-  (void)ctas_per_sm;
+cudaError_t launch_band(const BandArgs &a, int smem_bytes, cudaStream_t st) {
   const bool fwd = a.warp_mode == DIBR_WARP_FORWARD;
-  // the stereo set (left, right, anaglyph) and the anaglyph alone, with 16-byte aligned
-  // rows: instances of their own
-  if (a.depth_src == DS_BINOM5 && fwd && a.fast_store) {
-    // bands of a few rows do not repay a CTA's tensor-memory allocation
-    const bool tm = a.row1 - a.row0 >= kTmemMinRows * a.grid;
+  // the stereo set (left, right, anaglyph) and the anaglyph alone: instances of their own
+  if (a.depth_src == DS_BINOM5 && fwd && a.out_mode != OM_BYTES) {
     if (a.outputs == kSetStereo)
-      return tm ? launch_band_t<DS_BINOM5, true, kSetStereo, true>(a, smem_bytes, st)
-                : launch_band_t<DS_BINOM5, true, kSetStereo, false>(a, smem_bytes, st);
+      return a.ragged ? launch_fixed<kSetStereo, true>(a, smem_bytes, st) : launch_fixed<kSetStereo, false>(a, smem_bytes, st);
     if (a.outputs == kSetAnaglyph)
-      return tm ? launch_band_t<DS_BINOM5, true, kSetAnaglyph, true>(a, smem_bytes, st)
-                : launch_band_t<DS_BINOM5, true, kSetAnaglyph, false>(a, smem_bytes, st);
+      return a.ragged ? launch_fixed<kSetAnaglyph, true>(a, smem_bytes, st) : launch_fixed<kSetAnaglyph, false>(a, smem_bytes, st);
   }
-  switch (a.depth_src) {
-    case DS_BINOM5: return fwd ? launch_band_t<DS_BINOM5, true>(a, smem_bytes, st) : launch_band_t<DS_BINOM5, false>(a, smem_bytes, st);
-    case DS_LUMA: return fwd ? launch_band_t<DS_LUMA, true>(a, smem_bytes, st) : launch_band_t<DS_LUMA, false>(a, smem_bytes, st);
-    default: return fwd ? launch_band_t<DS_GLOBAL, true>(a, smem_bytes, st) : launch_band_t<DS_GLOBAL, false>(a, smem_bytes, st);
-  }
+  return a.ragged ? launch_any<true>(a, smem_bytes, st) : launch_any<false>(a, smem_bytes, st);
 }
 
-template <uint32_t OUTS>
+template <uint32_t OUTS, bool RAG>
 static cudaError_t launch_batch_t(const BatchArgs &b, int grid, int smem_bytes, bool chained, cudaStream_t st) {
   static std::atomic<uint64_t> done{0};
-  cudaError_t e = allow_smem(batch_kernel<OUTS>, done);
+  cudaError_t e = allow_smem(batch_kernel<OUTS, RAG>, done);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
@@ -1204,14 +1457,19 @@ static cudaError_t launch_batch_t(const BatchArgs &b, int grid, int smem_bytes, 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained ? 1 : 0;
-  e = cudaLaunchKernelEx(&cfg, batch_kernel<OUTS>, b);
+  e = cudaLaunchKernelEx(&cfg, batch_kernel<OUTS, RAG>, b);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_batch(const BatchArgs &b, int grid, int smem_bytes, bool chained, cudaStream_t st) {
-  if (b.outs == kSetStereo) return launch_batch_t<kSetStereo>(b, grid, smem_bytes, chained, st);
-  if (b.outs == kSetAnaglyph) return launch_batch_t<kSetAnaglyph>(b, grid, smem_bytes, chained, st);
-  return launch_batch_t<0>(b, grid, smem_bytes, chained, st);
+  if (b.outs == kSetStereo)
+    return b.ragged ? launch_batch_t<kSetStereo, true>(b, grid, smem_bytes, chained, st)
+                    : launch_batch_t<kSetStereo, false>(b, grid, smem_bytes, chained, st);
+  if (b.outs == kSetAnaglyph)
+    return b.ragged ? launch_batch_t<kSetAnaglyph, true>(b, grid, smem_bytes, chained, st)
+                    : launch_batch_t<kSetAnaglyph, false>(b, grid, smem_bytes, chained, st);
+  return b.ragged ? launch_batch_t<0, true>(b, grid, smem_bytes, chained, st)
+                  : launch_batch_t<0, false>(b, grid, smem_bytes, chained, st);
 }
 
 }  // namespace dibr

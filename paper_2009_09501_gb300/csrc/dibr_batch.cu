@@ -38,8 +38,16 @@ static int batch_zguard(const dibr_params *p, int n_params) {
   return g;
 }
 
+// An image's shape for the launch plans.
+static BatchShape shape_of(const dibr_image &im, const dibr_params &p, const dibr_outputs &o) {
+  const uint8_t *out[O_COUNT];
+  for (int k = 0; k < O_COUNT; ++k) out[k] = out_slot(o, k);
+  return BatchShape{im.width, im.height, zchunks_of(im.width, out_mode_of(p.outputs, out, o.pitch)),
+                    rows_aligned(im.rgb, im.pitch)};
+}
+
 void dibr_ctx::release_batch_buffers() {
-  for (DevBuf *b : {&batch_desc, &batch_img, &batch_depth}) {
+  for (DevBuf *b : {&batch_desc, &batch_depth}) {
     dev_free(b->ptr);
     b->ptr = nullptr;
     b->bytes = 0;
@@ -67,15 +75,15 @@ dibr_status dibr_ctx::enqueue_batch_device(int n, const dibr_image *imgs, const 
                                            const dibr_outputs *outs) {
   if (n == 0) return DIBR_OK;
   std::vector<int> own, shared;
-  const BatchLimits lim{max_smem, smem_per_sm, tuning.ring_slots, tuning.ctas_per_sm, batch_zguard(p, n_params)};
+  const BatchLimits lim{{max_smem, smem_per_sm, tuning.ring_slots, tuning.ctas_per_sm}, batch_zguard(p, n_params)};
   for (int i = 0; i < n; ++i) {
-    const int w = imgs[i].width, rb = round_up(3 * w, 16);
+    const BatchShape shape = shape_of(imgs[i], p[n_params == 1 ? 0 : i], outs[i]);
     int cl = 0;
     BatchClass c[1];
-    const bool fits = plan_batch_classes(1, &w, &rb, lim, &cl, c) == 1;
+    const bool fits = plan_batch_classes(1, &shape, lim, &cl, c) == 1;
     const int64_t slots = static_cast<int64_t>(num_sms) * (fits ? c[0].per : 1);
     bool big = fits && tuning.rows_per_unit == 0 && imgs[i].height >= kOwnLaunchRows * slots;
-    const auto t = class_tune.find(block_of(w));
+    const auto t = class_tune.find(block_of(shape));
     if (fits && tuning.rows_per_unit == 0 && t != class_tune.end() && t->second.own >= 0) big = t->second.own == 1;
     (big ? own : shared).push_back(i);
   }
@@ -110,64 +118,37 @@ dibr_status dibr_ctx::enqueue_grouped(int n, const dibr_image *imgs, const dibr_
                                       const dibr_outputs *outs) {
   prev_band = false;
   if (n == 0) return DIBR_OK;
-  // --- inputs that a bulk row copy cannot read directly are repacked (16-byte rows)
-  std::vector<const uint8_t *> in(n);
-  std::vector<int64_t> in_pitch(n);
-  std::vector<int> row_bytes(n);
-  size_t realign_bytes = 0, depth_bytes = 0;
-  for (int i = 0; i < n; ++i) {
-    const dibr_image &im = imgs[i];
-    const bool ok = (reinterpret_cast<uintptr_t>(im.rgb) & 15u) == 0 && (im.pitch & 15) == 0 && (3 * im.width) % 16 == 0;
-    if (!ok) realign_bytes += static_cast<size_t>(round_up(3 * im.width, 16)) * im.height;
+  // --- cross-bilateral depths first, into one buffer
+  size_t depth_bytes = 0;
+  for (int i = 0; i < n; ++i)
     if (p[n_params == 1 ? 0 : i].depth_rule == DIBR_DEPTH_LUMA_XBF)
-      depth_bytes += static_cast<size_t>(round_up(im.width, 16)) * im.height;
-  }
+      depth_bytes += static_cast<size_t>(round_up(imgs[i].width, 16)) * imgs[i].height;
   dibr_status s;
-  if (realign_bytes && (s = ensure(batch_img, realign_bytes)) != DIBR_OK) return s;
   if (depth_bytes && (s = ensure(batch_depth, depth_bytes)) != DIBR_OK) return s;
-  size_t ro = 0, dof = 0;
+  size_t dof = 0;
   std::vector<const uint8_t *> depth_in(n, nullptr);
   std::vector<int64_t> depth_pitch_in(n, 0);
   for (int i = 0; i < n; ++i) {
     const dibr_image &im = imgs[i];
     const dibr_params &pp = p[n_params == 1 ? 0 : i];
-    const bool ok = (reinterpret_cast<uintptr_t>(im.rgb) & 15u) == 0 && (im.pitch & 15) == 0 && (3 * im.width) % 16 == 0;
-    if (ok) {
-      in[i] = im.rgb;
-      in_pitch[i] = im.pitch;
-      row_bytes[i] = 3 * im.width;
-    } else {
-      const int64_t ap = round_up(3 * im.width, 16);
-      uint8_t *dst = batch_img.ptr + ro;
-      cudaError_t e = cudaMemcpy2DAsync(dst, ap, im.rgb, im.pitch, 3 * static_cast<size_t>(im.width), im.height,
-                                        cudaMemcpyDeviceToDevice, stream);
-      if (e != cudaSuccess) return cuda_fail(e, "repacking a batch input");
-      in[i] = dst;
-      in_pitch[i] = ap;
-      row_bytes[i] = static_cast<int>(ap);  // whole 16-byte units; the padding is never used
-      ro += static_cast<size_t>(ap) * im.height;
-    }
-    if (pp.depth_rule == DIBR_DEPTH_LUMA_XBF) {
-      const int64_t dp = round_up(im.width, 16);
-      uint8_t *dd = batch_depth.ptr + dof;
-      cudaError_t e = launch_xbf(in[i], in_pitch[i], im.width, im.height, pp.xbf_radius, pp.xbf_sigma_s,
-                                 pp.xbf_sigma_r, dd, dp, stream);
-      if (e != cudaSuccess) return cuda_fail(e, "cross-bilateral launch");
-      ++launches;
-      depth_in[i] = dd;
-      depth_pitch_in[i] = dp;
-      dof += static_cast<size_t>(dp) * im.height;
-    }
+    if (pp.depth_rule != DIBR_DEPTH_LUMA_XBF) continue;
+    const int64_t dp = round_up(im.width, 16);
+    uint8_t *dd = batch_depth.ptr + dof;
+    cudaError_t e = launch_xbf(im.rgb, im.pitch, im.width, im.height, pp.xbf_radius, pp.xbf_sigma_s, pp.xbf_sigma_r, dd,
+                               dp, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "cross-bilateral launch");
+    ++launches;
+    depth_in[i] = dd;
+    depth_pitch_in[i] = dp;
+    dof += static_cast<size_t>(dp) * im.height;
   }
   // --- one launch per group of images of equal block width, widest first
-  std::vector<int> widths(n), heights(n), class_of(n), order(n);
-  for (int i = 0; i < n; ++i) {
-    widths[i] = imgs[i].width;
-    heights[i] = imgs[i].height;
-  }
+  std::vector<BatchShape> shapes(n);
+  std::vector<int> class_of(n), order(n);
+  for (int i = 0; i < n; ++i) shapes[i] = shape_of(imgs[i], p[n_params == 1 ? 0 : i], outs[i]);
   BatchClass cls[kMaxClasses];
-  const BatchLimits lim{max_smem, smem_per_sm, tuning.ring_slots, tuning.ctas_per_sm, batch_zguard(p, n_params)};
-  const int nclass = plan_batch_classes(n, widths.data(), row_bytes.data(), lim, class_of.data(), cls);
+  const BatchLimits lim{{max_smem, smem_per_sm, tuning.ring_slots, tuning.ctas_per_sm}, batch_zguard(p, n_params)};
+  const int nclass = plan_batch_classes(n, shapes.data(), lim, class_of.data(), cls);
   if (nclass < 1) {
     set_error("batch images too wide for shared memory");
     return DIBR_E_INVALID;
@@ -177,12 +158,12 @@ dibr_status dibr_ctx::enqueue_grouped(int n, const dibr_image *imgs, const dibr_
     const auto t = class_tune.find(cls[c].nc);
     if (t == class_tune.end()) continue;
     BatchLimits l2 = lim;
-    if (lim.ring_slots == 0 && t->second.nb > 0) l2.ring_slots = t->second.nb;
-    if (lim.ctas_per_sm == 0 && t->second.per > 0) l2.ctas_per_sm = t->second.per;
+    if (lim.band.ring_slots == 0 && t->second.nb > 0) l2.band.ring_slots = t->second.nb;
+    if (lim.band.ctas_per_sm == 0 && t->second.per > 0) l2.band.ctas_per_sm = t->second.per;
     if (!plan_class(cls[c], l2)) plan_class(cls[c], lim);
   }
-  order_by_area(n, widths.data(), heights.data(), order.data());
-  plan_unit_rows(n, heights.data(), class_of.data(), nclass, num_sms, tuning.rows_per_unit, cls);
+  order_by_area(n, shapes.data(), order.data());
+  plan_unit_rows(n, shapes.data(), class_of.data(), nclass, num_sms, tuning.rows_per_unit, cls);
   if (tuning.rows_per_unit == 0)
     for (int c = 0; c < nclass; ++c) {
       const auto t = class_tune.find(cls[c].nc);
@@ -222,8 +203,8 @@ dibr_status dibr_ctx::enqueue_grouped(int n, const dibr_image *imgs, const dibr_
     const dibr_outputs &o = outs[i];
     ImageDesc &d = descs[i];
     std::memset(&d, 0, sizeof(d));
-    d.in = in[i];
-    d.in_pitch = in_pitch[i];
+    d.in = im.rgb;
+    d.in_pitch = im.pitch;
     d.depth_in = depth_in[i];
     d.depth_in_pitch = depth_pitch_in[i];
     for (int k = 0; k < O_COUNT; ++k) d.out[k] = out_slot(o, k);
@@ -232,17 +213,21 @@ dibr_status dibr_ctx::enqueue_grouped(int n, const dibr_image *imgs, const dibr_
     d.W = im.width;
     d.H = im.height;
     d.nch = chunks_of(im.width);
-    d.row_bytes = row_bytes[i];
+    d.nchz = shapes[i].nchz;
+    d.row_bytes = 3 * im.width;
     d.outputs = pp.outputs;
+    d.out_mode = out_mode_of(pp.outputs, d.out, o.pitch);
     d.warp_mode = pp.warp_mode;
     d.depth_src = pp.depth_rule == DIBR_DEPTH_LUMA_BINOM5 ? DS_BINOM5 : pp.depth_rule == DIBR_DEPTH_LUMA ? DS_LUMA : DS_GLOBAL;
     shift_tables(&pp, d.lut_h, d.lut_n);
   }
   // every image of one fixed output set: the launches use that set's kernel instance
   uint32_t fixed = 0;
+  bool ragged = false;
   for (int i = 0; i < n; ++i) {
     const ImageDesc &d = descs[i];
-    const uint32_t f = fixed_set(d.outputs, d.depth_src, d.warp_mode, d.out, d.out_pitch);
+    const uint32_t f = fixed_set(d.outputs, d.depth_src, d.warp_mode, d.out_mode);
+    ragged |= !shapes[i].aligned || d.out_mode != OM_ALIGNED || maps_ragged(d.outputs, d.out, d.depth_pitch);
     fixed = i == 0 ? f : (f == fixed ? fixed : 0u);
   }
   int u = 0;
@@ -271,9 +256,11 @@ dibr_status dibr_ctx::enqueue_grouped(int n, const dibr_image *imgs, const dibr_
     b.nb = cls[c].nb;
     b.srow = cls[c].srow;
     b.nch_max = cls[c].nch_max;
+    b.nchz_max = cls[c].nchz_max;
     b.nc = cls[c].nc;
     b.zguard = lim.zguard;
     b.outs = fixed;
+    b.ragged = ragged;
     const int grid = std::max(1, std::min(cls[c].n_units, num_sms * cls[c].per));
     e = launch_batch(b, grid, cls[c].smem, c > 0, stream);
     if (e != cudaSuccess) return cuda_fail(e, "batch kernel launch");
@@ -336,7 +323,7 @@ dibr_status dibr_autotune_batch(dibr_ctx *c, int n, const dibr_image *imgs, cons
   cudaSetDevice(c->device);
   // the images of each size class (block width), timed alone under every candidate plan
   std::map<int, std::vector<int>> groups;
-  for (int i = 0; i < n; ++i) groups[block_of(imgs[i].width)].push_back(i);
+  for (int i = 0; i < n; ++i) groups[block_of(shape_of(imgs[i], p[n_params == 1 ? 0 : i], outs[i]))].push_back(i);
   std::vector<ClassTune> cands;
   cands.push_back(ClassTune{0, 0, 0, 1});  // a band launch per image
   for (int rows : {0, 2, 4, 8, 16, 32, 64})

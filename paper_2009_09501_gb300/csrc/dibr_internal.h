@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
+
 #include "dibr.h"
 
 namespace dibr {
@@ -30,6 +32,14 @@ enum LoadMode : int {
   LM_BULK = 1,   // one contiguous bulk copy (cp.async.bulk) per row
   LM_T3 = 2,     // 3-D tensor {inner, 3W/inner, H}, boxes {inner, step, 1} (cp.async.bulk.tensor)
   LM_T2 = 3      // 2-D tensor {3W, H}, boxes {256, 1}: any width
+};
+
+// How a launch's RGB output rows meet 16-byte boundaries (the host decides per image).
+enum OutMode : int {
+  OM_ALIGNED = 0,  // every row starts on one (or no RGB output is requested)
+  OM_SHIFT = 1,    // all outputs' rows start equally far from one: chunks are shifted onto it
+  OM_HALF = 2,     // the side-by-side frame alone: each half's chunks shifted to 8-byte boundaries
+  OM_BYTES = 3     // anything else: byte stores
 };
 
 // Bits of the device status word.
@@ -75,6 +85,7 @@ struct BandArgs {
   int32_t srow;      // bytes per ring slot
   int32_t nb;        // ring slots
   int32_t nch;       // 16-pixel chunks per row
+  int32_t nchz;      // 16-target chunks per z-buffer row (one more where chunks are shifted)
   int32_t nc;        // threads per CTA, one 16-pixel chunk each (multiple of 32)
   int32_t zguard;    // guard targets on each side of a z-buffer row (>= the largest shift)
   int32_t grid;      // CTAs; CTA b owns rows row0 + [b*n/grid, (b+1)*n/grid), n = row1 - row0
@@ -84,7 +95,8 @@ struct BandArgs {
   uint32_t outputs;  // DIBR_OUT_* bits
   int32_t warp_mode; // DIBR_WARP_*
   int32_t depth_src; // DepthSource
-  int32_t fast_store;  // every RGB output base and the output pitch are 16-byte aligned
+  int32_t out_mode;  // OutMode
+  int32_t ragged;    // some input or output row does not start on a 16-byte boundary
   int *status;
   unsigned long long timeout_ns;
   int32_t lut_h[256];  // low 16 bits: hL[d], high 16 bits: hR[d] (signed)
@@ -93,21 +105,22 @@ struct BandArgs {
 
 // Shared-memory layout of the band kernel (bytes from the dynamic smem base).
 //   bar   ring-slot mbarriers full[kMaxRing]
-//   flags +0: the batch's current work unit; +8, +16: the per-row mbarriers (every warp
-//         has scattered the row / has published its summary and cleared its targets)
-//   lut   uint2 per value of 255 - depth: byte offsets of the left / right target
+//   flags +0: the batch's current work unit; +8, +24: the per-row mbarriers (every warp has
+//         written the row's targets / has published its summary and cleared its targets);
+//         +48: the tensor-memory base
+//   lut   uint2 per value of 255 - depth: byte offsets of the left / right target (gather:
+//         the shifts)
 //   wsum  per row parity, view and warp: {has a filled target, first, last filled entry}
 //   ring  input rows;  drow  255 - depth of the current row, one byte per column
 //   zb    z-buffers, [parity][view] rows of zlen targets separated by zguard guard targets
-//         (targets a shift moves outside the row land in a guard and are never read);
-//         the literal gather keeps int32 lut_n[256] here instead
+//         (targets a shift moves outside the row land in a guard and are never read)
 struct BandSmem {
   int bar, flags, lut, wsum, ring, drow, zb, zstride, total;
 };
 
 __host__ __device__ inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
-__host__ __device__ inline BandSmem band_smem_layout(int nb, int srow, int nch, int nwarps, int zguard) {
+__host__ __device__ inline BandSmem band_smem_layout(int nb, int srow, int nch, int nchz, int nwarps, int zguard) {
   BandSmem s;
   s.bar = 0;
   s.flags = 8 * kMaxRing;
@@ -116,10 +129,9 @@ __host__ __device__ inline BandSmem band_smem_layout(int nb, int srow, int nch, 
   s.ring = round_up(s.wsum + 2 * 2 * nwarps * 16, 128);
   s.drow = round_up(s.ring + nb * srow, 16);
   s.zb = round_up(s.drow + nch * kChunk, 16);
-  const int zlen = nch * kChunk;  // a multiple of 16 targets: rows stay 16-byte aligned
-  s.zstride = zlen + zguard;      // words from one row's target 0 to the next row's
-  const int zbytes = 4 * (4 * zlen + 5 * zguard);
-  s.total = s.zb + (zbytes > 1024 ? zbytes : 1024);
+  const int zlen = nchz * kChunk;  // a multiple of 16 targets: rows stay 16-byte aligned
+  s.zstride = zlen + zguard;       // words from one row's target 0 to the next row's
+  s.total = s.zb + 4 * (4 * zlen + 5 * zguard);
   return s;
 }
 
@@ -143,9 +155,9 @@ struct alignas(16) ImageDesc {
   int64_t depth_in_pitch;
   uint8_t *out[O_COUNT];
   int64_t out_pitch, depth_pitch;
-  int32_t W, H, nch, row_bytes;
+  int32_t W, H, nch, nchz, row_bytes;
   uint32_t outputs;
-  int32_t warp_mode, depth_src, pad;
+  int32_t warp_mode, depth_src, out_mode, pad[3];
   int32_t lut_h[256];
   int32_t lut_n[256];
 };
@@ -161,22 +173,63 @@ struct BatchArgs {
   int *counter;
   int *status;
   unsigned long long timeout_ns;
-  int32_t nb, srow, nch_max, nc, zguard;
+  int32_t nb, srow, nch_max, nchz_max, nc, zguard;
   uint32_t outs;  // kSetStereo / kSetAnaglyph: every image is of that kind (fixed_set); 0: any
+  int32_t ragged;  // some image's rows are not on 16-byte boundaries
 };
 
 // Output sets with kernel instances of their own (outputs fixed at compile time): binomial
-// depth, forward warp, and every requested RGB output and the output pitch 16-byte aligned.
+// depth, forward warp, whole-word stores.
 constexpr uint32_t kSetStereo = DIBR_OUT_ANAGLYPH | DIBR_OUT_LEFT | DIBR_OUT_RIGHT;
 constexpr uint32_t kSetAnaglyph = DIBR_OUT_ANAGLYPH;
 
 // The fixed set an image belongs to (kSetStereo, kSetAnaglyph), else 0.
-inline uint32_t fixed_set(uint32_t outputs, int depth_src, int warp_mode, const uint8_t *const *out, int64_t pitch) {
-  if (depth_src != DS_BINOM5 || warp_mode != DIBR_WARP_FORWARD) return 0u;
-  if (outputs != kSetStereo && outputs != kSetAnaglyph) return 0u;
-  const uintptr_t bits = reinterpret_cast<uintptr_t>(out[O_ANA]) | reinterpret_cast<uintptr_t>(out[O_LEFT]) |
-                         reinterpret_cast<uintptr_t>(out[O_RIGHT]) | static_cast<uintptr_t>(pitch);
-  return (bits & 15u) == 0 ? outputs : 0u;
+inline uint32_t fixed_set(uint32_t outputs, int depth_src, int warp_mode, int out_mode) {
+  if (depth_src != DS_BINOM5 || warp_mode != DIBR_WARP_FORWARD || out_mode == OM_BYTES) return 0u;
+  return outputs == kSetStereo || outputs == kSetAnaglyph ? outputs : 0u;
+}
+
+// How an image's RGB outputs meet 16-byte boundaries.
+inline int out_mode_of(uint32_t outputs, const uint8_t *const *out, int64_t pitch) {
+  const uint32_t rgb = outputs & (DIBR_OUT_ANAGLYPH | DIBR_OUT_LEFT | DIBR_OUT_RIGHT | DIBR_OUT_HSBS);
+  if (!rgb) return OM_ALIGNED;
+  uintptr_t first = 0;
+  bool any = false, same = true;
+  for (int i = 0; i < O_COUNT; ++i) {
+    if (!(rgb & kOutBits[i])) continue;
+    const uintptr_t r = reinterpret_cast<uintptr_t>(out[i]) & 15u;
+    same = same && (!any || r == first);
+    first = r;
+    any = true;
+  }
+  if (same && first == 0 && (pitch & 15) == 0) return OM_ALIGNED;
+  if (rgb == DIBR_OUT_HSBS && !(outputs & DIBR_OUT_HOLES)) return OM_HALF;
+  return same && !(rgb & DIBR_OUT_HSBS) ? OM_SHIFT : OM_BYTES;
+}
+
+// Some requested depth or holes row does not start on a 16-byte boundary.
+inline bool maps_ragged(uint32_t outputs, const uint8_t *const *out, int64_t depth_pitch) {
+  uintptr_t bits = 0;
+  for (int i : {static_cast<int>(O_DEPTH), static_cast<int>(O_HOLES)})
+    if (outputs & kOutBits[i]) bits |= reinterpret_cast<uintptr_t>(out[i]) | static_cast<uintptr_t>(depth_pitch);
+  return (bits & 15u) != 0;
+}
+
+// Input rows that all start on 16-byte boundaries.
+inline bool rows_aligned(const uint8_t *p, int64_t pitch) {
+  return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (pitch & 15) == 0;
+}
+
+inline int chunks_of(int width) { return (width + kChunk - 1) / kChunk; }
+// Chunks of a z-buffer row: shifted by up to 15 columns in the modes that shift.
+inline int zchunks_of(int width, int out_mode) {
+  return out_mode == OM_SHIFT || out_mode == OM_HALF ? chunks_of(width + kChunk - 1) : chunks_of(width);
+}
+// Bytes of a ring slot: the 16-byte units a row touches, and what the luminance's loads of
+// whole chunks reach.
+inline int slot_bytes(int width, bool aligned) {
+  const int row = round_up(3 * width + (aligned ? 0 : 15), 16), chunks = 48 * chunks_of(width);
+  return round_up(row > chunks ? row : chunks, 128);
 }
 
 // ---- planning a batch (host; no allocation, so the no-allocation entry point shares it)
@@ -187,11 +240,40 @@ inline uint32_t fixed_set(uint32_t outputs, int depth_src, int warp_mode, const 
 // images are grouped by block width and each group gets a launch of its own plan; the
 // launches follow one another on the stream, widest first, each allowed to start while
 // the previous one finishes its last units (programmatic dependent launch).
-constexpr int kMaxClasses = 16;  // distinct block widths: 32 .. 480 threads in steps of 32
+constexpr int kMaxClasses = 16;  // distinct block widths: 32 .. 512 threads in steps of 32
+
+// The plan of a block: ring depth, CTAs per SM and shared memory.
+struct BandPlan {
+  int nb, per, smem;
+};
+
+// What bounds a plan: device limits and the tuning's caps (0: none).
+struct BandLimits {
+  int max_smem, smem_per_sm;
+  int ring_slots, ctas_per_sm;
+};
+
+// The deepest ring at the most CTAs per SM within the limits (128 registers per thread: the
+// kernels' launch bound; 2048 threads per SM).  Returns false if no plan fits.
+inline bool plan_smem(BandPlan &p, const BandLimits &lim, int nc, int srow, int nch, int nchz, int zguard, int min_nb) {
+  const int max_nb = lim.ring_slots <= 0 ? kMaxRing : lim.ring_slots < min_nb ? min_nb : lim.ring_slots < kMaxRing ? lim.ring_slots : kMaxRing;
+  const int by_regs = 65536 / (nc * 128), by_threads = 2048 / nc;
+  p = BandPlan{0, 0, 0};
+  for (int nb = min_nb; nb <= max_nb; ++nb) {
+    const int tot = band_smem_layout(nb, srow, nch, nchz, nc / 32, zguard).total;
+    if (tot > lim.max_smem) continue;
+    int per = lim.smem_per_sm / (tot + 1024);
+    if (per > by_regs) per = by_regs;
+    if (per > by_threads) per = by_threads;
+    if (lim.ctas_per_sm > 0 && per > lim.ctas_per_sm) per = lim.ctas_per_sm;
+    if (per >= 1 && per >= p.per) p = BandPlan{nb, per, tot};
+  }
+  return p.per >= 1;
+}
 
 struct BatchClass {
   int nc;          // threads per block
-  int nch_max;     // 16-column chunks of the widest row in the group
+  int nch_max, nchz_max;  // 16-column chunks of the widest row in the group (source, z-buffer)
   int srow;        // bytes per ring slot
   int nb, per;     // ring slots; CTAs per SM
   int smem;        // dynamic shared memory per block
@@ -200,62 +282,51 @@ struct BatchClass {
 };
 
 struct BatchLimits {
-  int max_smem, smem_per_sm;  // device limits
-  int ring_slots, ctas_per_sm;  // tuning caps (0: none)
+  BandLimits band;
   int zguard;                   // z-buffer guard of every image of the batch (the largest)
 };
 
-inline int chunks_of(int width) { return (width + kChunk - 1) / kChunk; }
-inline int block_of(int width) { return round_up(chunks_of(width), 32); }
+// An image as the planning sees it.
+struct BatchShape {
+  int width, height, nchz;
+  bool aligned;  // input rows on 16-byte boundaries
+};
 
-// Ring depth and CTAs per SM of one group (nc, nch_max and srow set): the deepest ring at
-// the most CTAs per SM within the limits.  Returns false if no plan fits.
+inline int block_of(const BatchShape &s) { return round_up(s.nchz, 32); }
+
+// The plan of one group (nc, chunks and srow set).  Returns false if no plan fits.
 inline bool plan_class(BatchClass &k, const BatchLimits &lim) {
-  const int max_nb = lim.ring_slots > 0 ? (lim.ring_slots < 4 ? 4 : lim.ring_slots < kMaxRing ? lim.ring_slots : kMaxRing)
-                                        : kMaxRing;
-  const int by_regs = 65536 / (k.nc * 128), by_threads = 2048 / k.nc;
-  const int max_per = by_regs < by_threads ? by_regs : by_threads;
-  k.per = 0;
-  for (int nb = 4; nb <= max_nb; ++nb) {
-    const int tot = band_smem_layout(nb, k.srow, k.nch_max, k.nc / 32, lim.zguard).total;
-    if (tot > lim.max_smem) continue;
-    int per = lim.smem_per_sm / (tot + 1024);
-    if (per > max_per) per = max_per;
-    if (lim.ctas_per_sm > 0 && per > lim.ctas_per_sm) per = lim.ctas_per_sm;
-    if (per >= 1 && per >= k.per) {  // the deepest ring at the best CTAs per SM
-      k.per = per;
-      k.nb = nb;
-    }
-  }
-  if (k.per < 1) return false;
-  k.smem = band_smem_layout(k.nb, k.srow, k.nch_max, k.nc / 32, lim.zguard).total;
+  BandPlan p;
+  if (!plan_smem(p, lim.band, k.nc, k.srow, k.nch_max, k.nchz_max, lim.zguard, 4)) return false;
+  k.nb = p.nb;
+  k.per = p.per;
+  k.smem = p.smem;
   return true;
 }
 
 // Groups the n images by block width (widest first), plans each group's ring and CTAs per
 // SM, and sets class_of[i].  Returns the number of groups, or -1 if some group fits no plan.
-inline int plan_batch_classes(int n, const int *width, const int *row_bytes, const BatchLimits &lim,
-                              int *class_of, BatchClass *cls) {
+inline int plan_batch_classes(int n, const BatchShape *shape, const BatchLimits &lim, int *class_of, BatchClass *cls) {
   int nclass = 0;
   for (int i = 0; i < n; ++i) {
-    const int nc = block_of(width[i]);
+    const int nc = block_of(shape[i]);
     int c = 0;
     while (c < nclass && cls[c].nc > nc) ++c;
     if (c == nclass || cls[c].nc != nc) {
       if (nclass == kMaxClasses) return -1;
       for (int k = nclass; k > c; --k) cls[k] = cls[k - 1];
-      cls[c] = BatchClass{nc, 1, 128, 4, 0, 0, 0, 0, 0};
+      cls[c] = BatchClass{nc, 1, 1, 128, 4, 0, 0, 0, 0, 0};
       ++nclass;
     }
   }
   for (int i = 0; i < n; ++i) {
     int c = 0;
-    while (cls[c].nc != block_of(width[i])) ++c;
+    while (cls[c].nc != block_of(shape[i])) ++c;
     class_of[i] = c;
-    const int nch = chunks_of(width[i]);
-    const int need = row_bytes[i] > 48 * nch ? row_bytes[i] : 48 * nch;
+    const int nch = chunks_of(shape[i].width), slot = slot_bytes(shape[i].width, shape[i].aligned);
     if (nch > cls[c].nch_max) cls[c].nch_max = nch;
-    if (round_up(need, 128) > cls[c].srow) cls[c].srow = round_up(need, 128);
+    if (shape[i].nchz > cls[c].nchz_max) cls[c].nchz_max = shape[i].nchz;
+    if (slot > cls[c].srow) cls[c].srow = slot;
   }
   for (int c = 0; c < nclass; ++c)
     if (!plan_class(cls[c], lim)) return -1;
@@ -269,7 +340,7 @@ inline int plan_batch_classes(int n, const int *width, const int *row_bytes, con
 // unit recomputes the two rows of context above it, so units are not made smaller than
 // needed.
 constexpr int kUnitRows = 32;
-inline void plan_unit_rows(int n, const int *height, const int *class_of, int nclass, int sms, int rows,
+inline void plan_unit_rows(int n, const BatchShape *shape, const int *class_of, int nclass, int sms, int rows,
                            BatchClass *cls) {
   for (int c = 0; c < nclass; ++c) {
     if (rows > 0) {
@@ -278,7 +349,7 @@ inline void plan_unit_rows(int n, const int *height, const int *class_of, int nc
     }
     int64_t total = 0;
     for (int i = 0; i < n; ++i)
-      if (class_of[i] == c) total += height[i];
+      if (class_of[i] == c) total += shape[i].height;
     const int64_t slots = static_cast<int64_t>(sms) * (cls[c].per > 0 ? cls[c].per : 1);
     cls[c].rows = total <= slots * kUnitRows ? static_cast<int>((total + slots - 1) / slots) : kUnitRows;
     if (cls[c].rows < 1) cls[c].rows = 1;
@@ -286,11 +357,12 @@ inline void plan_unit_rows(int n, const int *height, const int *class_of, int nc
 }
 
 // order[0..n) = image indices, largest area first (stable insertion sort, no allocation)
-inline void order_by_area(int n, const int *width, const int *height, int *order) {
+inline void order_by_area(int n, const BatchShape *shape, int *order) {
+  auto area = [&](int i) { return static_cast<int64_t>(shape[i].width) * shape[i].height; };
   for (int i = 0; i < n; ++i) {
-    const int64_t a = static_cast<int64_t>(width[i]) * height[i];
+    const int64_t a = area(i);
     int k = i;
-    while (k > 0 && static_cast<int64_t>(width[order[k - 1]]) * height[order[k - 1]] < a) {
+    while (k > 0 && area(order[k - 1]) < a) {
       order[k] = order[k - 1];
       --k;
     }
@@ -314,7 +386,7 @@ struct InpaintArgs {
 };
 
 // Host launchers (dibr_band.cu, dibr_xbf.cu, dibr_inpaint.cu).
-cudaError_t launch_band(const BandArgs &a, int smem_bytes, int ctas_per_sm, cudaStream_t st);
+cudaError_t launch_band(const BandArgs &a, int smem_bytes, cudaStream_t st);
 // chained: may start while the previous launch on the stream finishes (the previous
 // launch is a batch launch of the same call).
 cudaError_t launch_batch(const BatchArgs &b, int grid, int smem_bytes, bool chained, cudaStream_t st);

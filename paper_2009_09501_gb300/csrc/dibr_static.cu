@@ -100,12 +100,13 @@ extern "C" dibr_status dibr_synthesize_batch_static(int n, const dibr_image *img
                                                     int n_params, const dibr_outputs *outs, void *cuda_stream) {
   if (n < 1 || n > kStaticMaxImages || !imgs || !p || !outs || (n_params != 1 && n_params != n))
     return DIBR_E_INVALID;
-  int widths[kStaticMaxImages], heights[kStaticMaxImages], row_bytes[kStaticMaxImages];
+  BatchShape shapes[kStaticMaxImages];
   for (int i = 0; i < n; ++i) {
     if (!valid_image(&p[n_params == 1 ? 0 : i], &imgs[i], &outs[i])) return DIBR_E_INVALID;
-    widths[i] = imgs[i].width;
-    heights[i] = imgs[i].height;
-    row_bytes[i] = 3 * imgs[i].width;
+    const uint8_t *out[O_COUNT];
+    for (int k = 0; k < O_COUNT; ++k) out[k] = out_slot(outs[i], k);
+    shapes[i] = BatchShape{imgs[i].width, imgs[i].height,
+                           zchunks_of(imgs[i].width, out_mode_of(p[n_params == 1 ? 0 : i].outputs, out, outs[i].pitch)), true};
   }
 
   int dev = 0;
@@ -130,15 +131,15 @@ extern "C" dibr_status dibr_synthesize_batch_static(int n, const dibr_image *img
     const int g = zguard_of(lh);
     if (g > zguard) zguard = g;
   }
-  const BatchLimits lim{d.max_smem, d.smem_per_sm, 0, 0, zguard};
-  const int nclass = plan_batch_classes(n, widths, row_bytes, lim, class_of, cls);
+  const BatchLimits lim{{d.max_smem, d.smem_per_sm, 0, 0}, zguard};
+  const int nclass = plan_batch_classes(n, shapes, lim, class_of, cls);
   if (nclass < 1) return DIBR_E_INVALID;
-  order_by_area(n, widths, heights, order);
+  order_by_area(n, shapes, order);
   // rows per unit as for the context's batches, larger while the unit list would not fit
-  plan_unit_rows(n, heights, class_of, nclass, d.sms, 0, cls);
+  plan_unit_rows(n, shapes, class_of, nclass, d.sms, 0, cls);
   auto count_units = [&]() {
     int64_t u = 0;
-    for (int i = 0; i < n; ++i) u += (heights[i] + cls[class_of[i]].rows - 1) / cls[class_of[i]].rows;
+    for (int i = 0; i < n; ++i) u += (shapes[i].height + cls[class_of[i]].rows - 1) / cls[class_of[i]].rows;
     return u;
   };
   while (count_units() > kStaticMaxUnits)
@@ -163,17 +164,20 @@ extern "C" dibr_status dibr_synthesize_batch_static(int n, const dibr_image *img
     dd.W = im.width;
     dd.H = im.height;
     dd.nch = chunks_of(im.width);
+    dd.nchz = shapes[i].nchz;
     dd.row_bytes = 3 * im.width;
     dd.outputs = pp.outputs;
+    dd.out_mode = out_mode_of(pp.outputs, dd.out, o.pitch);
     dd.warp_mode = pp.warp_mode;
     dd.depth_src = pp.depth_rule == DIBR_DEPTH_LUMA_BINOM5 ? DS_BINOM5 : DS_LUMA;
     shift_tables(&pp, dd.lut_h, dd.lut_n);
   }
   // every image of one fixed output set: the launches use that set's kernel instance
   uint32_t fixed = 0;
+  bool ragged = false;
   for (int i = 0; i < n; ++i) {
-    const uint32_t f = fixed_set(descs[i].outputs, descs[i].depth_src, descs[i].warp_mode, descs[i].out,
-                                 descs[i].out_pitch);
+    const uint32_t f = fixed_set(descs[i].outputs, descs[i].depth_src, descs[i].warp_mode, descs[i].out_mode);
+    ragged |= descs[i].out_mode != OM_ALIGNED || maps_ragged(descs[i].outputs, descs[i].out, descs[i].depth_pitch);
     fixed = i == 0 ? f : (f == fixed ? fixed : 0u);
   }
   int n_units = 0;
@@ -204,9 +208,11 @@ extern "C" dibr_status dibr_synthesize_batch_static(int n, const dibr_image *img
     b.nb = cls[c].nb;
     b.srow = cls[c].srow;
     b.nch_max = cls[c].nch_max;
+    b.nchz_max = cls[c].nchz_max;
     b.nc = cls[c].nc;
     b.zguard = zguard;
     b.outs = fixed;
+    b.ragged = ragged;
     const int grid = cls[c].n_units < d.sms * cls[c].per ? cls[c].n_units : d.sms * cls[c].per;
     e = launch_batch(b, grid > 0 ? grid : 1, cls[c].smem, c > 0, stream);
     if (e != cudaSuccess) return DIBR_E_CUDA;
