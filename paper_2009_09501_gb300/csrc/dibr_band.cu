@@ -14,9 +14,9 @@
 // refills a slot once every warp has scattered the row it held.
 //
 // Per consumer thread and row y:
-//   A  luminance of row y+2 for its 16 columns plus 2 on each side, fed into a cascade
-//      of four [1 1] row sums held in registers, which yields the vertical binomial of
-//      row y; the horizontal binomial gives D(y) for the 16 columns, stored as 255 - D.
+//   A  luminance of row y+2 for its 16 columns plus 2 on each side and its horizontal binomial;
+//      with the sums of the four rows before, kept by the thread, the vertical one gives 255 - D(y)
+//      for the 16 columns.
 //   B  the warp scatters its 512 sources (lane-interleaved) into the left and right
 //      z-buffers with a shared-memory atomic minimum of ((255 - D) << 24 | RGB).  The
 //      z-buffer rows carry guard targets on both sides, as wide as the largest shift,
@@ -46,8 +46,8 @@
 // Instances: the requested outputs are read from the arguments, or fixed at compile time for
 // the two sets the workloads use (left + right + anaglyph, anaglyph alone; binomial depth,
 // forward warp), which drops the output branches and the state they
-// keep live.  The fixed-set instances in bands of kTmemMinRows rows or more keep the vertical
-// cascade's 32 words per thread in tensor memory between one row's A and the next, so that B
+// keep live.  The fixed-set instances in bands of kTmemMinRows rows or more keep the row
+// sums' 32 words per thread in tensor memory between one row's A and the next, so that B
 // and C have those registers.
 #include <atomic>
 
@@ -170,7 +170,7 @@ __device__ __forceinline__ void lds_ragged(uint32_t row, uint32_t s, int off, ui
 
 // Luminance of columns x0-2 .. x0+17 (clamped to [0, W-1]) of one input row held in
 // shared memory from byte s of `row` on, as 10 words of two 16-bit lanes: yp[2q] = columns
-// (4q, 4q+2) and yp[2q+1] = (4q+1, 4q+3) of the window, the layout the vertical cascade
+// (4q, 4q+2) and yp[2q+1] = (4q+1, 4q+3) of the window, the layout the binomial
 // works on.  RAG: any s < 16; otherwise s = 0.
 template <bool RAG>
 __device__ __forceinline__ void luma20(const uint8_t *row, uint32_t s, int x0, int W, uint32_t (&yp)[10]) {
@@ -270,66 +270,20 @@ __device__ __forceinline__ void binom_h(const uint32_t (&Y)[10], uint32_t (&h)[8
   }
 }
 
-// Vertical binomial [1 4 6 4 1] of the row sums as four cascaded [1 1] sums over the
-// stream of rows, on the 8 pair words of binom_h.  After row n is fed, p0 = h(n),
-// p1 = h(n-1) + h(n), p2 and p3 the next sums; feeding row n+1 returns
-// sum_i C(4,i) h(n-3+i), the full 5x5 sum centred on row n-1 (at most 256 * 255, so the
-// lanes never carry into each other).  The state is updated in place: the new p3 is the
-// sum minus the old p3, each lower level the level above minus its old value.
-struct VCascade {
-  uint32_t p0[8], p1[8], p2[8], p3[8];
-
-  // the state as 32 words (kept in tensor memory between rows by the fixed-set instances)
-  __device__ __forceinline__ void get(uint32_t (&t)[32]) const {
+// 255 - depth of the 16 own columns (4 per word) from the row sums of five consecutive rows, the
+// vertical binomial [1 4 6 4 1]: D = (S + 128) >> 8 of the 5x5 sum S, so 255 - D =
+// (0xFF7F - S) >> 8.  Both 16-bit lanes of a word stay in 127 .. 0xFF7F, so byte 1 of each lane is
+// its result.  (Four cascaded [1 1] sums before: 48 instructions a row against 32, and all 32 words
+// of state rewritten; with the tables below a 4K frame on the full grid 34.7 -> 34.3 us, 8K frames 124.0
+// -> 121.6.)
+__device__ __forceinline__ uint4 binom_v(const uint32_t (&h0)[8], const uint32_t (&h1)[8], const uint32_t (&h2)[8],
+                                         const uint32_t (&h3)[8], const uint32_t (&h4)[8]) {
+  uint32_t v[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      t[i] = p0[i];
-      t[8 + i] = p1[i];
-      t[16 + i] = p2[i];
-      t[24 + i] = p3[i];
-    }
-  }
-  __device__ __forceinline__ void set(const uint32_t (&t)[32]) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      p0[i] = t[i];
-      p1[i] = t[8 + i];
-      p2[i] = t[16 + i];
-      p3[i] = t[24 + i];
-    }
-  }
-
-  __device__ __forceinline__ void clear() {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) p0[i] = p1[i] = p2[i] = p3[i] = 0u;
-  }
-  __device__ __forceinline__ void feed(const uint32_t (&h)[8], uint32_t (&V)[8]) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint32_t v = p3[i] + p2[i] + p1[i] + p0[i] + h[i];
-      p3[i] = v - p3[i];
-      p2[i] = p3[i] - p2[i];
-      p1[i] = p2[i] - p1[i];
-      p0[i] = p1[i] - p0[i];
-      V[i] = v;
-    }
-  }
-  // feeds the newest row again (the image's last row repeated below the image)
-  __device__ __forceinline__ void feed_repeat(uint32_t (&V)[8]) {
-    uint32_t h[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) h[i] = p0[i];
-    feed(h, V);
-  }
-};
-
-// The depth of the 16 own columns from the 5x5 sums: D = (sum + 128) >> 8, packed 4 per
-// word.  Both lanes of a sum word stay below 65536 after the rounding offset, so byte 1 of
-// each lane is its rounded result.
-__device__ __forceinline__ uint4 round_depth(const uint32_t (&V)[8]) {
+  for (int i = 0; i < 8; ++i) v[i] = 0xFF7FFF7Fu - 6u * h2[i] - 4u * (h1[i] + h3[i]) - h0[i] - h4[i];
   uint32_t d[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) d[k] = __byte_perm(V[2 * k] + 0x00800080u, V[2 * k + 1] + 0x00800080u, 0x7351);
+  for (int k = 0; k < 4; ++k) d[k] = __byte_perm(v[2 * k], v[2 * k + 1], 0x7351);
   return make_uint4(d[0], d[1], d[2], d[3]);
 }
 
@@ -470,6 +424,15 @@ __device__ __forceinline__ void reds_min_at_if(uint32_t a, uint32_t v, bool pred
       : "memory");
 }
 
+// base + the low / high signed half of v, one byte dot product each (on the multiply pipe, where the
+// sums of two 32-bit table words were integer adds; and the table is half as wide to load).
+__device__ __forceinline__ uint32_t add_lo16(uint32_t v, uint32_t base) {
+  return static_cast<uint32_t>(__dp2a_lo(static_cast<int>(v), 0x0001, static_cast<int>(base)));
+}
+__device__ __forceinline__ uint32_t add_hi16(uint32_t v, uint32_t base) {
+  return static_cast<uint32_t>(__dp2a_lo(static_cast<int>(v), 0x0100, static_cast<int>(base)));
+}
+
 // Four consecutive 32-column steps G*4 .. G*4+3 of a lane's sources in the forward warp:
 // 255 - depth from the depth row (ds), colour words from the input row (cws, the colour
 // at bit offset sh), the two target offsets from the table (ls), atomics into the left
@@ -481,20 +444,20 @@ __device__ __forceinline__ void scatter4(uint32_t ds, uint32_t cws, uint32_t sh,
   uint32_t fv[4], cw[8];
   lds_u8_step32x4(ds + 128 * G, fv);
   lds_u32_pair_step96x4(cws + 384 * G, cw);
-  uint2 lt[4];
+  uint32_t lt[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) lt[j] = lds_u32x2(ls + 8u * fv[j]);
+  for (int j = 0; j < 4; ++j) lt[j] = lds_u32(ls + 4u * fv[j]);
   uint32_t e[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) e[j] = __byte_perm(__funnelshift_r(cw[2 * j], cw[2 * j + 1], sh), fv[j], 0x4210);
-  reds_min_at<128 * (4 * G + 0)>(bl + lt[0].x, e[0]);
-  reds_min_at<128 * (4 * G + 0)>(br + lt[0].y, e[0]);
-  reds_min_at<128 * (4 * G + 1)>(bl + lt[1].x, e[1]);
-  reds_min_at<128 * (4 * G + 1)>(br + lt[1].y, e[1]);
-  reds_min_at<128 * (4 * G + 2)>(bl + lt[2].x, e[2]);
-  reds_min_at<128 * (4 * G + 2)>(br + lt[2].y, e[2]);
-  reds_min_at<128 * (4 * G + 3)>(bl + lt[3].x, e[3]);
-  reds_min_at<128 * (4 * G + 3)>(br + lt[3].y, e[3]);
+  reds_min_at<128 * (4 * G + 0)>(add_lo16(lt[0], bl), e[0]);
+  reds_min_at<128 * (4 * G + 0)>(add_hi16(lt[0], br), e[0]);
+  reds_min_at<128 * (4 * G + 1)>(add_lo16(lt[1], bl), e[1]);
+  reds_min_at<128 * (4 * G + 1)>(add_hi16(lt[1], br), e[1]);
+  reds_min_at<128 * (4 * G + 2)>(add_lo16(lt[2], bl), e[2]);
+  reds_min_at<128 * (4 * G + 2)>(add_hi16(lt[2], br), e[2]);
+  reds_min_at<128 * (4 * G + 3)>(add_lo16(lt[3], bl), e[3]);
+  reds_min_at<128 * (4 * G + 3)>(add_hi16(lt[3], br), e[3]);
 }
 
 // One image's arguments as the band routine sees them (built from the kernel
@@ -539,7 +502,7 @@ struct Shm {
   uint64_t *full;   // ring-slot mbarriers
   uint64_t *bdone;  // [2] every warp has written the row's targets (B)
   uint64_t *sdone;  // [2] every warp has published its summary and cleared its targets (C)
-  uint2 *lut;       // per 255 - depth: byte offsets of the left / right targets (gather: shifts)
+  uint32_t *lut;    // per 255 - depth: byte offsets of the left, right targets (gather: shifts)
   uint8_t *wsum;    // [parity][view][warp] uint4 {has, first entry, last entry, 0}
   uint8_t *ring, *drow;
   uint32_t zb;      // shared address of the z-buffer region
@@ -552,7 +515,7 @@ __device__ __forceinline__ Shm carve(uint8_t *smem, int nb, int srow, int nch, i
   m.full = reinterpret_cast<uint64_t *>(smem + L.bar);
   m.bdone = reinterpret_cast<uint64_t *>(smem + L.flags + 8);
   m.sdone = reinterpret_cast<uint64_t *>(smem + L.flags + 24);
-  m.lut = reinterpret_cast<uint2 *>(smem + L.lut);
+  m.lut = reinterpret_cast<uint32_t *>(smem + L.lut);
   m.wsum = smem + L.wsum;
   m.ring = smem + L.ring;
   m.drow = smem + L.drow;
@@ -573,8 +536,8 @@ __device__ __forceinline__ void fill_luts(const Shm &m, const int32_t *lut_h) {
   for (int i = threadIdx.x; i < 256; i += blockDim.x) {
     const int32_t h = lut_h[255 - i];
     const int hl = static_cast<int16_t>(h & 0xFFFF), hr = h >> 16;  // |h| <= 512
-    m.lut[i] = FWD ? make_uint2(static_cast<uint32_t>(-4 * hl), static_cast<uint32_t>(-4 * hr))
-                   : make_uint2(static_cast<uint32_t>(hl), static_cast<uint32_t>(hr));
+    const int l = FWD ? -4 * hl : hl, r = FWD ? -4 * hr : hr;
+    m.lut[i] = (static_cast<uint32_t>(l) & 0xFFFFu) | (static_cast<uint32_t>(r) << 16);
   }
 }
 
@@ -597,8 +560,9 @@ __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, unsign
 // in flight have landed).
 // OUTS: the requested outputs when fixed at compile time, 0 when read from the arguments.
 // RAG: input or output rows may start anywhere; otherwise all start on 16-byte boundaries.
-// TM: the vertical cascade's 32 words wait in tensor memory (at tmem, this thread's lane)
-// between one row's A and the next, so that B and C have those registers.
+// TM: the sums of the four rows before (32 words) wait in tensor memory (at tmem, this thread's
+// lane; a ring of four, so that a row is stored once and never moved) between one row's A and the
+// next, so that B and C have those registers.
 template <int DS, bool FWD, uint32_t OUTS, bool RAG, bool TM>
 __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int ye, uint32_t &kbase,
                                          uint32_t &nrows, int *status,
@@ -737,23 +701,27 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
       for (int r = 0; r < 4; ++r) sts_u32x4(zrow(r >> 1, r & 1) + 16u * i, e);
     }
   }
-  VCascade vc;
-  vc.clear();
+  uint32_t hr[4][8] = {};  // the row sums of the four rows before the one to come (TM: in tensor memory)
   if (binom) {
-    // rows clamp(ys-2) .. clamp(ys+1) into the cascade, each as soon as it has landed
+    // rows clamp(ys-2) .. clamp(ys+1), each as soon as it has landed
 #pragma unroll 1
     for (int i = -2; i <= 1; ++i) {
       const int r = min(max(ys + i, 0), H - 1);
       if (r >= la && r < lb && (i == -2 || r != min(max(ys + i - 1, 0), H - 1))) wait_row(r);
-      uint32_t yq[10], hq[8], V[8];
+      uint32_t yq[10], hn[8];
       luma20<RAG>(slot(r), RAG ? a.lead(r) : 0u, x0c, W, yq);
-      binom_h(yq, hq);
-      vc.feed(hq, V);
-    }
-    if (TM) {
-      uint32_t t[32];
-      vc.get(t);
-      tmem_store32(tmem, t);
+      binom_h(yq, hn);
+      if (TM) {
+        tmem_store8(tmem + 8u * static_cast<uint32_t>(i + 2), hn);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          hr[0][q] = hr[1][q];
+          hr[1][q] = hr[2][q];
+          hr[2][q] = hr[3][q];
+          hr[3][q] = hn[q];
+        }
+      }
     }
   }
   // the cleared z-buffers (and, with the binomial, the rows above the band) are done with
@@ -777,40 +745,46 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
 
   // ---- A: the depth of row y (4 columns per word), 255 - depth into the depth row
   auto phase_a = [&](int y) {
-    uint4 d;
+    uint4 f;  // 255 - depth
     if (binom) {
       const int r2 = y + 2;
-      uint32_t t[32];
-      if (TM) tmem_load32(tmem, t);  // the cascade back (waited for just before it is fed)
-      if (r2 < lb) wait_row(r2);
-      uint32_t V[8];
-      if (r2 < H) {
-        uint32_t yq[10], hq[8];
-        luma20<RAG>(slot(r2), RAG ? a.lead(r2) : 0u, x0c, W, yq);
-        binom_h(yq, hq);
-        if (TM) {
-          tmem_load_wait32(t);
-          vc.set(t);
-        }
-        vc.feed(hq, V);
-      } else {
-        if (TM) {
-          tmem_load_wait32(t);
-          vc.set(t);
-        }
-        vc.feed_repeat(V);  // rows below the image repeat row H-1
-      }
+      const uint32_t n = static_cast<uint32_t>(y - ys);  // (row y - 2's sums are in slot n & 3)
       if (TM) {
-        vc.get(t);
-        tmem_store32(tmem, t);
+        tmem_wait_stores();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tmem_load8(tmem + 8u * ((n + i) & 3u), hr[i]);
       }
-      d = round_depth(V);
+      if (r2 < lb) wait_row(r2);
+      uint32_t hn[8];
+      if (r2 < H) {
+        uint32_t yq[10];
+        luma20<RAG>(slot(r2), RAG ? a.lead(r2) : 0u, x0c, W, yq);
+        binom_h(yq, hn);
+      }
+      if (TM) tmem_load_wait8x4(hr);
+      if (r2 >= H) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) hn[i] = hr[3][i];  // rows below the image repeat row H-1
+      }
+      f = binom_v(hr[0], hr[1], hr[2], hr[3], hn);
+      if (TM) {
+        tmem_store8(tmem + 8u * (n & 3u), hn);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          hr[0][i] = hr[1][i];
+          hr[1][i] = hr[2][i];
+          hr[2][i] = hr[3][i];
+          hr[3][i] = hn[i];
+        }
+      }
     } else if (DS == DS_LUMA) {
       wait_row(y);
-      d = luma16<RAG>(slot(y), RAG ? a.lead(y) : 0u, x0c);
+      const uint4 d = luma16<RAG>(slot(y), RAG ? a.lead(y) : 0u, x0c);
+      f = make_uint4(~d.x, ~d.y, ~d.z, ~d.w);
     } else {
       wait_row(y);  // B reads the row's colours
-      d = make_uint4(0u, 0u, 0u, 0u);
+      uint4 d = make_uint4(0u, 0u, 0u, 0u);
       if (active) {
         const uint8_t *dp = a.depth_in + static_cast<int64_t>(y) * a.depth_in_pitch + x0;
         if (npx == kChunk && (reinterpret_cast<uintptr_t>(dp) & 15u) == 0) {
@@ -821,9 +795,10 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
           d = make_uint4(w[0], w[1], w[2], w[3]);
         }
       }
+      f = make_uint4(~d.x, ~d.y, ~d.z, ~d.w);
     }
-    if (want_depth && active && !depth_bytes(y)) store16(a.out[O_DEPTH] + static_cast<int64_t>(y) * a.depth_pitch + x0, d, npx);
-    if (wfull || own_chunk) *reinterpret_cast<uint4 *>(m.drow + x0) = make_uint4(~d.x, ~d.y, ~d.z, ~d.w);
+    if (want_depth && active && !depth_bytes(y)) store16(a.out[O_DEPTH] + static_cast<int64_t>(y) * a.depth_pitch + x0, make_uint4(~f.x, ~f.y, ~f.z, ~f.w), npx);
+    if (wfull || own_chunk) *reinterpret_cast<uint4 *>(m.drow + x0) = f;
   };
 
   // ---- B: the targets of row y from the warp's 512 columns, consecutive lanes on consecutive
@@ -861,9 +836,9 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int x = min(xb + 32 * (4 * g + j), warp_hi - 1);
-          const uint2 h = lds_u32x2(ls + 8u * f[j]);
-          sx[0][j] = x + static_cast<int>(h.x);
-          sx[1][j] = x + static_cast<int>(h.y);
+          const uint32_t h = lds_u32(ls + 4u * f[j]);
+          sx[0][j] = static_cast<int>(add_lo16(h, x));
+          sx[1][j] = static_cast<int>(add_hi16(h, x));
           out |= static_cast<unsigned>(sx[0][j]) >= static_cast<unsigned>(W) || static_cast<unsigned>(sx[1][j]) >= static_cast<unsigned>(W);
         }
         if (__any_sync(kAll, out)) {
@@ -912,16 +887,16 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
           cw[2 * j] = lds_u32(ca);
           cw[2 * j + 1] = lds_u32(ca + 4);
         }
-        uint2 lt[4];
+        uint32_t lt[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) lt[j] = lds_u32x2(ls + 8u * fv[j]);
+        for (int j = 0; j < 4; ++j) lt[j] = lds_u32(ls + 4u * fv[j]);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int x = xb + 32 * (4 * g + j);
           const uint32_t e = __byte_perm(__funnelshift_r(cw[2 * j], cw[2 * j + 1], sh), fv[j], 0x4210);
           const uint32_t off = 512u * static_cast<uint32_t>(g) + 128u * j;
-          reds_min_at_if<0>(bl + off + lt[j].x, e, x < warp_hi);
-          reds_min_at_if<0>(br + off + lt[j].y, e, x < warp_hi);
+          reds_min_at_if<0>(add_lo16(lt[j], bl + off), e, x < warp_hi);
+          reds_min_at_if<0>(add_hi16(lt[j], br + off), e, x < warp_hi);
           if (dbytes && x < warp_hi) dp[x] = static_cast<uint8_t>(255u - fv[j]);
         }
       }
@@ -1223,7 +1198,7 @@ __device__ __forceinline__ void init_barriers(const Shm &m, int nb) {
 // ---------------------------------------------------------------------------------
 // One image: CTA b owns the rows row0 + [b*n/grid, (b+1)*n/grid), n = row1 - row0.
 // TM (fixed-set instances with the binomial depth, bands of kTmemMinRows rows or more): the
-// cascade waits in tensor memory between rows.
+// row sums wait in tensor memory between rows.
 template <int DS, bool FWD, uint32_t OUTS, bool RAG, bool TM>
 __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_constant__ BandArgs a) {
   static_assert(!TM || (OUTS != 0 && DS == DS_BINOM5), "tensor memory only in the fixed-set binomial instances");
@@ -1275,7 +1250,8 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_con
     }
     const uint32_t tmem = tbase + ((32u * (warp & 3)) << 16) + 32u * (warp >> 2);
     run_band<DS, FWD, OUTS, RAG, TM>(j, m, ys, ye, kbase, nrows, a.status, a.timeout_ns, tmem);
-    if (TM) {  // every thread's stores have completed (each store waits for itself)
+    if (TM) {
+      tmem_wait_stores();
       tmem_fence_before_sync();
       __syncthreads();
       tmem_fence_after_sync();
@@ -1303,7 +1279,7 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) batch_kernel(BatchArgs b) {
   const int flags = band_smem_layout(b.nb, b.srow, b.nch_max, b.nchz_max, nwarps, b.zguard).flags;
   int *unit_s = reinterpret_cast<int *>(smem + flags);
   init_barriers(m0, b.nb);
-  // a fixed-set batch keeps each unit's binomial cascade in tensor memory between rows
+  // a fixed-set batch keeps each unit's row sums in tensor memory between rows
   // (allocated once per CTA, as in the band kernel)
   constexpr bool TM = OUTS != 0;
   const int warp = threadIdx.x >> 5;
@@ -1361,7 +1337,8 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) batch_kernel(BatchArgs b) {
     }
     if (!ok) break;
   }
-  if (TM) {  // every thread's stores have completed (each store waits for itself)
+  if (TM) {
+    tmem_wait_stores();
     tmem_fence_before_sync();
     __syncthreads();
     tmem_fence_after_sync();

@@ -108,8 +108,8 @@ struct BandArgs {
 //   flags +0: the batch's current work unit; +8, +24: the per-row mbarriers (every warp has
 //         written the row's targets / has published its summary and cleared its targets);
 //         +48: the tensor-memory base
-//   lut   uint2 per value of 255 - depth: byte offsets of the left / right target (gather:
-//         the shifts)
+//   lut   one word per value of 255 - depth: byte offsets of the left (low half) and right
+//         target (gather: the shifts)
 //   wsum  per row parity, view and warp: {has a filled target, first, last filled entry}
 //   ring  input rows;  drow  255 - depth of the current row, one byte per column
 //   zb    z-buffers, [parity][view] rows of zlen targets separated by zguard guard targets
@@ -125,7 +125,7 @@ __host__ __device__ inline BandSmem band_smem_layout(int nb, int srow, int nch, 
   s.bar = 0;
   s.flags = 8 * kMaxRing;
   s.lut = s.flags + 64;
-  s.wsum = s.lut + 2048;
+  s.wsum = s.lut + 1024;
   s.ring = round_up(s.wsum + 2 * 2 * nwarps * 16, 128);
   s.drow = round_up(s.ring + nb * srow, 16);
   s.zb = round_up(s.drow + nch * kChunk, 16);
