@@ -70,7 +70,7 @@ def whole_job_rate(units_per_rank, seconds_per_rank, world, dist=None, device="c
     return world * units_per_rank / reduce_max(seconds_per_rank, dist, device)
 
 
-BAND_SOURCES = ("dibr_band.cu", "dibr_internal.h", "dibr_ptx.cuh")
+BAND_SOURCES = ("dibr_band.cuh", "dibr_internal.h", "dibr_ptx.cuh")
 INPAINT_SOURCES = ("dibr_inpaint.cu", "dibr_internal.h", "dibr_ptx.cuh")
 XBF_SOURCES = ("dibr_xbf.cu", "dibr_internal.h", "dibr_ptx.cuh")
 

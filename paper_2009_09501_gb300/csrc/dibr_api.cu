@@ -250,6 +250,7 @@ dibr_status dibr_ctx::plan_band(int W, int H, int depth_src, const uint8_t *in, 
     return DIBR_E_INVALID;
   }
   a.nb = plan.nb;
+  a.zp = plan.zp;
   smem = plan.smem;
   per_sm = plan.per;
   a.grid = std::max(1, std::min(H, num_sms * per_sm));

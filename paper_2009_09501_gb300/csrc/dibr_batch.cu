@@ -259,6 +259,7 @@ dibr_status dibr_ctx::enqueue_grouped(int n, const dibr_image *imgs, const dibr_
     b.nchz_max = cls[c].nchz_max;
     b.nc = cls[c].nc;
     b.zguard = lim.zguard;
+    b.zp = cls[c].zp;
     b.outs = fixed;
     b.ragged = ragged;
     const int grid = std::max(1, std::min(cls[c].n_units, num_sms * cls[c].per));

@@ -87,6 +87,7 @@ struct BandArgs {
   int32_t nch;       // 16-pixel chunks per row
   int32_t nchz;      // 16-target chunks per z-buffer row (one more where chunks are shifted)
   int32_t nc;        // threads per CTA, one 16-pixel chunk each (multiple of 32)
+  int32_t zp;        // z-buffer rows per view: 2 used by alternate rows, or 1
   int32_t zguard;    // guard targets on each side of a z-buffer row (>= the largest shift)
   int32_t grid;      // CTAs; CTA b owns rows row0 + [b*n/grid, (b+1)*n/grid), n = row1 - row0
   int32_t row0, row1;  // the rows this launch computes (all of them: 0, H)
@@ -112,7 +113,7 @@ struct BandArgs {
 //         target (gather: the shifts)
 //   wsum  per row parity, view and warp: {has a filled target, first, last filled entry}
 //   ring  input rows;  drow  255 - depth of the current row, one byte per column
-//   zb    z-buffers, [parity][view] rows of zlen targets separated by zguard guard targets
+//   zb    z-buffers, [zp][view] rows of zlen targets separated by zguard guard targets
 //         (targets a shift moves outside the row land in a guard and are never read)
 struct BandSmem {
   int bar, flags, lut, wsum, ring, drow, zb, zstride, total;
@@ -120,7 +121,7 @@ struct BandSmem {
 
 __host__ __device__ inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
-__host__ __device__ inline BandSmem band_smem_layout(int nb, int srow, int nch, int nchz, int nwarps, int zguard) {
+__host__ __device__ inline BandSmem band_smem_layout(int nb, int srow, int nch, int nchz, int nwarps, int zguard, int zp) {
   BandSmem s;
   s.bar = 0;
   s.flags = 8 * kMaxRing;
@@ -131,7 +132,7 @@ __host__ __device__ inline BandSmem band_smem_layout(int nb, int srow, int nch, 
   s.zb = round_up(s.drow + nch * kChunk, 16);
   const int zlen = nchz * kChunk;  // a multiple of 16 targets: rows stay 16-byte aligned
   s.zstride = zlen + zguard;       // words from one row's target 0 to the next row's
-  s.total = s.zb + 4 * (4 * zlen + 5 * zguard);
+  s.total = s.zb + 4 * (2 * zp * zlen + (2 * zp + 1) * zguard);
   return s;
 }
 
@@ -173,7 +174,7 @@ struct BatchArgs {
   int *counter;
   int *status;
   unsigned long long timeout_ns;
-  int32_t nb, srow, nch_max, nchz_max, nc, zguard;
+  int32_t nb, srow, nch_max, nchz_max, nc, zguard, zp;
   uint32_t outs;  // kSetStereo / kSetAnaglyph: every image is of that kind (fixed_set); 0: any
   int32_t ragged;  // some image's rows are not on 16-byte boundaries
 };
@@ -242,9 +243,9 @@ inline int slot_bytes(int width, bool aligned) {
 // the previous one finishes its last units (programmatic dependent launch).
 constexpr int kMaxClasses = 16;  // distinct block widths: 32 .. 512 threads in steps of 32
 
-// The plan of a block: ring depth, CTAs per SM and shared memory.
+// The plan of a block: ring depth, z-buffer rows per view, CTAs per SM and shared memory.
 struct BandPlan {
-  int nb, per, smem;
+  int nb, zp, per, smem;
 };
 
 // What bounds a plan: device limits and the tuning's caps (0: none).
@@ -253,20 +254,26 @@ struct BandLimits {
   int ring_slots, ctas_per_sm;
 };
 
-// The deepest ring at the most CTAs per SM within the limits (128 registers per thread: the
-// kernels' launch bound; 2048 threads per SM).  Returns false if no plan fits.
+// The most CTAs per SM within the limits (128 registers per thread: the kernels' launch bound;
+// 2048 threads per SM), two z-buffer rows per view unless one leaves room for more CTAs (rows of
+// 3857 to 4096 pixels: two CTAs instead of one, a 4031 x 3023 frame 99 -> 66 us; 1080p: four instead of three, 10.3 -> 9.1), and the deepest ring.  Returns
+// false if no plan fits.
 inline bool plan_smem(BandPlan &p, const BandLimits &lim, int nc, int srow, int nch, int nchz, int zguard, int min_nb) {
   const int max_nb = lim.ring_slots <= 0 ? kMaxRing : lim.ring_slots < min_nb ? min_nb : lim.ring_slots < kMaxRing ? lim.ring_slots : kMaxRing;
   const int by_regs = 65536 / (nc * 128), by_threads = 2048 / nc;
-  p = BandPlan{0, 0, 0};
-  for (int nb = min_nb; nb <= max_nb; ++nb) {
-    const int tot = band_smem_layout(nb, srow, nch, nchz, nc / 32, zguard).total;
-    if (tot > lim.max_smem) continue;
-    int per = lim.smem_per_sm / (tot + 1024);
-    if (per > by_regs) per = by_regs;
-    if (per > by_threads) per = by_threads;
-    if (lim.ctas_per_sm > 0 && per > lim.ctas_per_sm) per = lim.ctas_per_sm;
-    if (per >= 1 && per >= p.per) p = BandPlan{nb, per, tot};
+  p = BandPlan{0, 0, 0, 0};
+  for (int zp = 2; zp >= 1; --zp) {
+    BandPlan q{0, zp, 0, 0};
+    for (int nb = min_nb; nb <= max_nb; ++nb) {
+      const int tot = band_smem_layout(nb, srow, nch, nchz, nc / 32, zguard, zp).total;
+      if (tot > lim.max_smem) continue;
+      int per = lim.smem_per_sm / (tot + 1024);
+      if (per > by_regs) per = by_regs;
+      if (per > by_threads) per = by_threads;
+      if (lim.ctas_per_sm > 0 && per > lim.ctas_per_sm) per = lim.ctas_per_sm;
+      if (per >= 1 && per >= q.per) q = BandPlan{nb, zp, per, tot};
+    }
+    if (q.per > p.per) p = q;
   }
   return p.per >= 1;
 }
@@ -275,7 +282,7 @@ struct BatchClass {
   int nc;          // threads per block
   int nch_max, nchz_max;  // 16-column chunks of the widest row in the group (source, z-buffer)
   int srow;        // bytes per ring slot
-  int nb, per;     // ring slots; CTAs per SM
+  int nb, zp, per; // ring slots, z-buffer rows per view, CTAs per SM
   int smem;        // dynamic shared memory per block
   int rows;        // rows per work unit
   int unit_begin, n_units;
@@ -299,6 +306,7 @@ inline bool plan_class(BatchClass &k, const BatchLimits &lim) {
   BandPlan p;
   if (!plan_smem(p, lim.band, k.nc, k.srow, k.nch_max, k.nchz_max, lim.zguard, 4)) return false;
   k.nb = p.nb;
+  k.zp = p.zp;
   k.per = p.per;
   k.smem = p.smem;
   return true;
@@ -315,7 +323,7 @@ inline int plan_batch_classes(int n, const BatchShape *shape, const BatchLimits 
     if (c == nclass || cls[c].nc != nc) {
       if (nclass == kMaxClasses) return -1;
       for (int k = nclass; k > c; --k) cls[k] = cls[k - 1];
-      cls[c] = BatchClass{nc, 1, 1, 128, 4, 0, 0, 0, 0, 0};
+      cls[c] = BatchClass{nc, 1, 1, 128, 4, 2, 0, 0, 0, 0, 0};
       ++nclass;
     }
   }
@@ -385,7 +393,10 @@ struct InpaintArgs {
                           // the next item to take (zeroed before the launch)
 };
 
-// Host launchers (dibr_band.cu, dibr_xbf.cu, dibr_inpaint.cu).
+// Host launchers (dibr_band*.cu, dibr_xbf.cu, dibr_inpaint.cu).
+cudaError_t launch_band_ragged(const BandArgs &a, int smem_bytes, cudaStream_t st);
+cudaError_t launch_band_any(const BandArgs &a, int smem_bytes, cudaStream_t st);
+cudaError_t launch_batch_any(const BatchArgs &b, int grid, int smem_bytes, bool chained, cudaStream_t st);
 cudaError_t launch_band(const BandArgs &a, int smem_bytes, cudaStream_t st);
 // chained: may start while the previous launch on the stream finishes (the previous
 // launch is a batch launch of the same call).

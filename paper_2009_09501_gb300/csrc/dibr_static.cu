@@ -211,6 +211,7 @@ extern "C" dibr_status dibr_synthesize_batch_static(int n, const dibr_image *img
     b.nchz_max = cls[c].nchz_max;
     b.nc = cls[c].nc;
     b.zguard = zguard;
+    b.zp = cls[c].zp;
     b.outs = fixed;
     b.ragged = ragged;
     const int grid = cls[c].n_units < d.sms * cls[c].per ? cls[c].n_units : d.sms * cls[c].per;
