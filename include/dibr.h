@@ -275,7 +275,7 @@ dibr_status dibr_synthesize_batch_static(int n, const dibr_image *imgs, const di
  *                  is small (one 4K frame: 8 rows), 32 rows otherwise;
  *   host_bands     row bands of dibr_synthesize_image with host input and outputs (the
  *                  bands' uploads, kernels and downloads overlap), 1..8; automatic: 4 from
- *                  2048 rows, 2 from 512, else 1;
+ *                  4 MB of input, else 1;
  *   frames_in_flight  1..16: when a frame is enqueued on the context's own stream while
  *                  earlier work is still queued there, and it shares no buffer with the
  *                  frame before it, its launch takes 1/n of the SM slots (in taller row

@@ -243,11 +243,17 @@ dibr_status dibr_ctx::plan_band(int W, int H, int depth_src, const uint8_t *in, 
   a.l2_prefetch = tuning.l2_prefetch == 1 ? 1 : 0;
   a.srow = std::max(slot_bytes(W, aligned), round_up(a.nbox * a.box_bytes, 128));
   a.depth_src = depth_src;
-  BandPlan plan;
-  const BandLimits lim{max_smem, smem_per_sm, tuning.ring_slots, tuning.ctas_per_sm};
-  if (!plan_smem(plan, lim, a.nc, a.srow, a.nch, a.nchz, zguard, depth_src == DS_BINOM5 ? 4 : 2)) {
-    set_error("width %d needs more shared memory than the device offers", W);
-    return DIBR_E_INVALID;
+  // (the plan of the last launch is kept: frames of one size follow one another, and at 4 us a
+  // small frame's launch its 0.2 us count)
+  const int key[8] = {a.nc, a.srow, a.nch, a.nchz, zguard, depth_src == DS_BINOM5 ? 4 : 2, tuning.ring_slots, tuning.ctas_per_sm};
+  if (std::memcmp(key, plan_key, sizeof(key)) != 0) {
+    plan_key[0] = 0;
+    const BandLimits lim{max_smem, smem_per_sm, tuning.ring_slots, tuning.ctas_per_sm};
+    if (!plan_smem(plan, lim, a.nc, a.srow, a.nch, a.nchz, zguard, key[5])) {
+      set_error("width %d needs more shared memory than the device offers", W);
+      return DIBR_E_INVALID;
+    }
+    std::memcpy(plan_key, key, sizeof(key));
   }
   a.nb = plan.nb;
   a.zp = plan.zp;
@@ -460,12 +466,37 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   return DIBR_OK;
 }
 
+dibr_status dibr_ctx::enqueue_rows(const dibr_image *img, const dibr_params *p, const dibr_outputs *o, int y0, int y1) {
+  prev_band = false;
+  BandArgs &a = args;
+  int smem = 0, per_sm = 1;
+  const int zguard = band_tables(p);
+  a.depth_in = nullptr;
+  a.depth_in_pitch = 0;
+  for (int i = 0; i < O_COUNT; ++i) a.out[i] = out_slot(*o, i);
+  a.out_pitch = o->pitch;
+  a.depth_pitch = o->depth_pitch;
+  a.outputs = p->outputs;
+  a.warp_mode = p->warp_mode;
+  dibr_status s = plan_band(img->width, img->height, p->depth_rule == DIBR_DEPTH_LUMA_BINOM5 ? DS_BINOM5 : DS_LUMA, img->rgb,
+                            img->pitch, zguard, a, smem, per_sm);
+  if (s == DIBR_OK) s = encode_input(a, img->rgb, img->pitch);
+  if (s != DIBR_OK) return s;
+  a.row0 = y0;
+  a.row1 = y1;
+  a.grid = std::max(1, std::min(y1 - y0, num_sms * per_sm));
+  const cudaError_t e = launch_band(a, smem, stream);
+  if (e != cudaSuccess) return cuda_fail(e, "band kernel launch");
+  ++launches;
+  return DIBR_OK;
+}
+
 dibr_status dibr_ctx::read_status() {
   prev_band = false;
-  int st = 0;
-  cudaError_t e = cudaMemcpyAsync(&st, status_dev, sizeof(int), cudaMemcpyDeviceToHost, stream);
+  cudaError_t e = cudaMemcpyAsync(status_host, status_dev, sizeof(int), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return cuda_fail(e, "synchronising the context stream");
+  const int st = *status_host;
   if (st) {
     cudaMemsetAsync(status_dev, 0, sizeof(int), stream);
     cudaStreamSynchronize(stream);
@@ -553,6 +584,11 @@ dibr_status dibr_create(const dibr_config *cfg_in, dibr_ctx **out) {
     c->owns_stream = true;
   }
   c->status_dev = static_cast<int *>(c->dev_alloc(64));
+  if (c->status_dev && cudaHostAlloc(reinterpret_cast<void **>(&c->status_host), 64, cudaHostAllocDefault) != cudaSuccess) {
+    cudaGetLastError();
+    c->dev_free(c->status_dev);
+    c->status_dev = nullptr;
+  }
   if (!c->status_dev) {
     if (c->owns_stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -561,6 +597,7 @@ dibr_status dibr_create(const dibr_config *cfg_in, dibr_ctx **out) {
   cudaMemsetAsync(c->status_dev, 0, 64, c->stream);
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) {
     c->dev_free(c->status_dev);
+    cudaFreeHost(c->status_host);
     if (c->owns_stream) cudaStreamDestroy(c->stream);
     delete c;
     return DIBR_E_CUDA;
@@ -577,6 +614,7 @@ void dibr_destroy(dibr_ctx *c) {
   c->release_buffers();
   c->dev_free(c->status_dev);
   cudaStreamSynchronize(c->stream);
+  cudaFreeHost(c->status_host);
   if (c->owns_stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -764,7 +802,9 @@ dibr_status dibr_ctx::synthesize_staged(const dibr_image *img, const dibr_params
   // row bands when both sides of the call are in host memory and every row band is
   // independent of the others' results (not with the 2-D fill or the cross-bilateral depth,
   // which need the whole frame first)
-  const int bands = tuning.host_bands > 0 ? std::min(tuning.host_bands, H) : H >= 2048 ? 4 : H >= 512 ? 2 : 1;
+  // (automatic: from 4 MB of input -- 1080p anaglyph 107 us in two bands, 102 in one, 95 in four, all
+  // three outputs 179, 171 and 173; 720p 104, 98 and 104)
+  const int bands = tuning.host_bands > 0 ? std::min(tuning.host_bands, H) : 3ll * W * H >= (4 << 20) ? std::min(4, H) : 1;
   if (bands > 1 && !img->on_device && !o->on_device && p->hole_fill == DIBR_FILL_ROW &&
       p->depth_rule != DIBR_DEPTH_LUMA_XBF)
     return synthesize_banded(img, p, o, bands);

@@ -47,6 +47,7 @@ struct dibr_ctx {
   int max_streams = 64;
   int max_batch = 256;
   int *status_dev = nullptr;
+  int *status_host = nullptr;  // its copy in pinned memory (read_status)
   unsigned long long timeout_ns = 2000000000ull;  // 2 s per bounded device-side wait
   dibr_tuning tuning{};      // zero fields: automatic
   std::map<int, dibr::ClassTune> class_tune;  // per block width: the autotuner's choices
@@ -61,6 +62,8 @@ struct dibr_ctx {
   // parameters {rule, P, T}; rebuilt only when a call brings others
   int32_t args_tables_key[3] = {-1, -1, -1};
   int args_zguard = 0;
+  int plan_key[8] = {};   // what the plan below was made for (dibr_api.cu plan_band)
+  dibr::BandPlan plan{};
   int band_tables(const dibr_params *p);  // fills args.lut_h / lut_n, returns the guard width
 
   // batched launches (dibr_batch.cu)
@@ -97,6 +100,8 @@ struct dibr_ctx {
                         dibr::BandArgs &a, int &smem, int &per_sm);
   dibr_status encode_input(dibr::BandArgs &a, const uint8_t *dev_rgb, int64_t pitch);
   dibr_status enqueue_device(const dibr_image *img, const dibr_params *p, const dibr_outputs *o);
+  // rows [y0, y1) of an image alone (not with the 2-D fill or the cross-bilateral depth)
+  dibr_status enqueue_rows(const dibr_image *img, const dibr_params *p, const dibr_outputs *o, int y0, int y1);
   dibr_status synthesize_staged(const dibr_image *img, const dibr_params *p, const dibr_outputs *o);
   dibr_status synthesize_banded(const dibr_image *img, const dibr_params *p, const dibr_outputs *o, int bands);
   void release_band_pipeline();

@@ -2,9 +2,9 @@
 //
 // Each open stream owns kSlots frame slots of resident device memory (input + requested
 // outputs).  dibr_submit_frame() queues a host frame.  A scheduler thread repeatedly
-// takes every queued frame that has a free slot (across all streams, up to max_batch),
-// uploads them on an H2D copy stream, runs them as one batched launch on the compute
-// stream once the uploads are done, and downloads the outputs on a D2H copy stream.  It
+// takes every queued frame that has a free slot (across all streams, up to max_batch) as a
+// batch and enqueues it in parts: a part's uploads on an H2D copy stream, its launch on the
+// compute stream once they are done, its downloads on a D2H copy stream.  It
 // does not wait for a batch to finish before forming the next one, so frames that arrive
 // while others are on the GPU join the next launch as soon as their stream has a free
 // slot.  A completion thread waits for each batch's download, stamps the completion
@@ -34,6 +34,8 @@ dibr_status check_image_args(const dibr_params *p, const dibr_image *img, const 
 
 constexpr int kSlots = 3;       // frames in flight per stream: upload, compute, download
 constexpr int kMaxQueued = 16;  // frames queued per stream beyond the slots
+constexpr size_t kPartBytes = 4u << 20;  // input bytes of a part of a batch (about 25 us of the host link)
+constexpr size_t kMaxParts = 4;          // row bands of one frame at most
 
 static uint64_t now_ns() {
   timespec t;
@@ -196,32 +198,69 @@ static void scheduler_loop(ServeState *st) {
     cudaMemsetAsync(status_word, 0, sizeof(int), st->gpu->stream);
     st->gpu->status_dev = status_word;
     st->gpu->timeout_ns = st->owner->timeout_ns;
-    st->gpu->prev_band = false;  // (the memset is other work on the stream)
-    for (size_t f = 0; f < b.frames.size(); ++f) {
-      const Frame &fr = b.meta[f];
-      if (cudaMemcpy2DAsync(const_cast<uint8_t *>(imgs[f].rgb), imgs[f].pitch, fr.in.rgb, fr.in.pitch,
-                            3 * static_cast<size_t>(imgs[f].width), imgs[f].height, cudaMemcpyHostToDevice,
-                            st->h2d) != cudaSuccess)
+    // Rows [y0, y1) of frame f up, or of its outputs down.
+    auto upload = [&](size_t f, int y0, int y1) {
+      const dibr_image &src = b.meta[f].in, &dst = imgs[f];
+      if (cudaMemcpy2DAsync(const_cast<uint8_t *>(dst.rgb) + y0 * dst.pitch, dst.pitch, src.rgb + y0 * src.pitch, src.pitch,
+                            3 * static_cast<size_t>(dst.width), y1 - y0, cudaMemcpyHostToDevice, st->h2d) != cudaSuccess)
         status = DIBR_E_CUDA;
-    }
-    cudaEventRecord(up, st->h2d);
-    cudaStreamWaitEvent(st->gpu->stream, up, 0);
-    if (status == DIBR_OK)
-      status = st->gpu->enqueue_batch_device(static_cast<int>(imgs.size()), imgs.data(), prms.data(),
-                                             static_cast<int>(prms.size()), outs.data());
-    cudaEventRecord(comp, st->gpu->stream);
-    cudaStreamWaitEvent(st->d2h, comp, 0);
-    for (size_t f = 0; f < b.frames.size() && status == DIBR_OK; ++f) {
-      const Frame &fr = b.meta[f];
+    };
+    auto download = [&](size_t f, int y0, int y1) {
+      const dibr_outputs &dst = b.meta[f].out, &src = outs[f];
       for (int k = 0; k < O_COUNT; ++k) {
         if (!(prms[f].outputs & bits[k])) continue;
-        const bool dep = is_map_output(k);
-        if (cudaMemcpy2DAsync(out_slot(fr.out, k), dep ? fr.out.depth_pitch : fr.out.pitch, out_slot(outs[f], k),
-                              dep ? outs[f].depth_pitch : outs[f].pitch,
-                              dep ? imgs[f].width : 3 * static_cast<size_t>(imgs[f].width), imgs[f].height,
-                              cudaMemcpyDeviceToHost, st->d2h) != cudaSuccess)
+        const bool map = is_map_output(k);
+        const int64_t dp = map ? dst.depth_pitch : dst.pitch, sp = map ? src.depth_pitch : src.pitch;
+        if (cudaMemcpy2DAsync(out_slot(dst, k) + y0 * dp, dp, out_slot(src, k) + y0 * sp, sp,
+                              map ? imgs[f].width : 3 * static_cast<size_t>(imgs[f].width), y1 - y0, cudaMemcpyDeviceToHost,
+                              st->d2h) != cudaSuccess)
           status = DIBR_E_CUDA;
       }
+    };
+    auto after_uploads = [&] {  // the compute stream goes on once the uploads so far are done
+      cudaEventRecord(up, st->h2d);
+      cudaStreamWaitEvent(st->gpu->stream, up, 0);
+      st->gpu->prev_band = false;
+    };
+    auto after_launch = [&] {  // ... and the downloads once its launches so far are
+      cudaEventRecord(comp, st->gpu->stream);
+      cudaStreamWaitEvent(st->d2h, comp, 0);
+    };
+    // The batch goes through the three streams in parts, so that one part's download runs beside
+    // the next one's upload (the host link bounds a batch; with the whole batch as one part, two
+    // 1080p and two 4K frames took 906 us, 547 in parts): small frames together, a launch for each
+    // part of at least kPartBytes of input, and a large frame by itself in row bands.
+    const size_t n = imgs.size();
+    for (size_t f = 0; f < n && status == DIBR_OK;) {
+      const size_t bytes = static_cast<size_t>(imgs[f].pitch) * imgs[f].height;
+      const int H = imgs[f].height;
+      const bool rows = prms[f].depth_rule != DIBR_DEPTH_LUMA_XBF;  // (its depth pass takes the whole frame)
+      const int bands = rows ? std::max(1, std::min(static_cast<int>(std::min<size_t>(kMaxParts, bytes / kPartBytes)), H / 8)) : 1;
+      if (bands > 1) {
+        auto row = [&](int j) { return static_cast<int>(static_cast<int64_t>(j) * H / bands); };
+        upload(f, 0, row(1));
+        for (int j = 0; j < bands && status == DIBR_OK; ++j) {
+          // (a band reads two rows past its own: they are in the next one's upload)
+          if (j + 1 < bands) upload(f, row(j + 1), row(j + 2));
+          after_uploads();
+          if (status == DIBR_OK) status = st->gpu->enqueue_rows(&imgs[f], &prms[f], &outs[f], row(j), row(j + 1));
+          after_launch();
+          if (status == DIBR_OK) download(f, row(j), row(j + 1));
+        }
+        ++f;
+        continue;
+      }
+      size_t end = f, sum = 0;
+      while (end < n && (end == f || sum < kPartBytes)) sum += static_cast<size_t>(imgs[end].pitch) * imgs[end].height, ++end;
+      for (size_t i = f; i < end; ++i) upload(i, 0, imgs[i].height);
+      after_uploads();
+      if (status == DIBR_OK)
+        status = end - f == 1 && rows ? st->gpu->enqueue_rows(&imgs[f], &prms[f], &outs[f], 0, H)
+                                      : st->gpu->enqueue_batch_device(static_cast<int>(end - f), &imgs[f], &prms[f],
+                                                                      static_cast<int>(end - f), &outs[f]);
+      after_launch();
+      for (size_t i = f; i < end && status == DIBR_OK; ++i) download(i, 0, imgs[i].height);
+      f = end;
     }
     cudaMemcpyAsync(&st->status_host[b.status_slot], status_word, sizeof(int), cudaMemcpyDeviceToHost, st->d2h);
     cudaEventRecord(b.done, st->d2h);
