@@ -239,7 +239,7 @@ dibr_status dibr_tuning_load(dibr_ctx *ctx, const char *path);
  * its back.  dibr_synthesize_batch needs a context, and creating one allocates; this entry
  * point needs none.  It calls no cudaMalloc, cudaFree or other allocating routine: the
  * small device scratch of the batched launch (a work counter, one descriptor per image, the
- * list of work units) lives in one fixed array of 267,008 bytes in the library's device
+ * list of work units) lives in one fixed array of 208,128 bytes in the library's device
  * data, which every GPU that loads the library holds until the process exits.
  *   - Inputs and outputs: device memory of the current device, as for dibr_enqueue_batch.
  *     Input rows must be whole 16-byte units: 16-byte aligned base and pitch, 3*width a

@@ -159,10 +159,14 @@ dibr_status check_image_args(const dibr_params *p, const dibr_image *img, const 
   return s;
 }
 
-// The kernels' packed tables: lut_h[d] = (hR << 16) | (hL & 0xFFFF); lut_n[d] = 510 * s_L(d).
-void shift_tables(const dibr_params *p, int32_t *lut_h, int32_t *lut_n) {
+// The kernels' packed tables: lut_h[d] = (hR << 16) | (hL & 0xFFFF); bit d of frac: s_L(d) is no
+// whole number.
+void shift_tables(const dibr_params *p, int32_t *lut_h, uint32_t *frac) {
   int16_t hL[256], hR[256];
-  build_tables(p, hL, hR, lut_n);
+  int32_t num[256];
+  build_tables(p, hL, hR, num);
+  for (int i = 0; i < 8; ++i) frac[i] = 0u;
+  for (int d = 0; d < 256; ++d) frac[d >> 5] |= static_cast<uint32_t>(num[d] % 510 != 0) << (d & 31);
   for (int d = 0; d < 256; ++d)
     lut_h[d] = static_cast<int32_t>((static_cast<uint32_t>(static_cast<uint16_t>(hR[d])) << 16) |
                                     static_cast<uint16_t>(hL[d]));
@@ -189,7 +193,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
 int dibr_ctx::band_tables(const dibr_params *p) {
   const int32_t key[3] = {p->disparity_rule, p->max_parallax_px, p->threshold};
   if (key[0] != args_tables_key[0] || key[1] != args_tables_key[1] || key[2] != args_tables_key[2]) {
-    shift_tables(p, args.lut_h, args.lut_n);
+    shift_tables(p, args.lut_h, args.frac);
     args_zguard = zguard_of(args.lut_h);
     for (int i = 0; i < 3; ++i) args_tables_key[i] = key[i];
   }

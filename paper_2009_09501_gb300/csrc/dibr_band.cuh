@@ -471,7 +471,7 @@ struct Job {
   const CUtensorMap *tmap;  // tensor-box load modes only
   const uint8_t *depth_in;
   int64_t depth_in_pitch;
-  const int32_t *lut_n;     // Fig. 3 gather: 510 * s_L(d)
+  const uint32_t *frac;     // Fig. 3 gather: bit d, s_L(d) is no whole number
   uint8_t *out[O_COUNT];
   int64_t out_pitch, depth_pitch;
   int W, H, nch, nchz, row_bytes, load_mode, nbox, box_bytes, box_step;
@@ -855,7 +855,7 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
 #pragma unroll
             for (int v = 0; v < 2; ++v)
               if (static_cast<unsigned>(sx[v][j]) >= static_cast<unsigned>(W))
-                sx[v][j] = sx[v][j] == -1 && a.lut_n[255u - f[j]] % 510 != 0 ? 0 : min(xb + 32 * (4 * g + j), warp_hi - 1);
+                sx[v][j] = sx[v][j] == -1 && (a.frac[(255u - f[j]) >> 5] >> ((255u - f[j]) & 31u) & 1u) ? 0 : min(xb + 32 * (4 * g + j), warp_hi - 1);
         }
         uint32_t c[2][4];
 #pragma unroll
@@ -1242,7 +1242,7 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_con
     j.tmap = &a.tmap;
     j.depth_in = a.depth_in;
     j.depth_in_pitch = a.depth_in_pitch;
-    j.lut_n = a.lut_n;
+    j.frac = a.frac;
 #pragma unroll
     for (int i = 0; i < O_COUNT; ++i) j.out[i] = a.out[i];
     j.out_pitch = a.out_pitch;
@@ -1329,7 +1329,7 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) batch_kernel(BatchArgs b) {
     j.tmap = nullptr;
     j.depth_in = dsc.depth_in;
     j.depth_in_pitch = dsc.depth_in_pitch;
-    j.lut_n = dsc.lut_n;
+    j.frac = dsc.frac;
 #pragma unroll
     for (int i = 0; i < O_COUNT; ++i) j.out[i] = dsc.out[i];
     j.out_pitch = dsc.out_pitch;

@@ -24,7 +24,7 @@ using namespace dibr;
 namespace dibr {
 dibr_status check_image_args(const dibr_params *p, const dibr_image *img, const dibr_outputs *o,
                              std::string *why);
-void shift_tables(const dibr_params *p, int32_t *lut_h, int32_t *lut_n);
+void shift_tables(const dibr_params *p, int32_t *lut_h, uint32_t *frac);
 }  // namespace dibr
 
 // The z-buffer guard every image of a batch fits in: the largest shift of their tables.
@@ -219,7 +219,7 @@ dibr_status dibr_ctx::enqueue_grouped(int n, const dibr_image *imgs, const dibr_
     d.out_mode = out_mode_of(pp.outputs, d.out, o.pitch);
     d.warp_mode = pp.warp_mode;
     d.depth_src = pp.depth_rule == DIBR_DEPTH_LUMA_BINOM5 ? DS_BINOM5 : pp.depth_rule == DIBR_DEPTH_LUMA ? DS_LUMA : DS_GLOBAL;
-    shift_tables(&pp, d.lut_h, d.lut_n);
+    shift_tables(&pp, d.lut_h, d.frac);
   }
   // every image of one fixed output set: the launches use that set's kernel instance
   uint32_t fixed = 0;

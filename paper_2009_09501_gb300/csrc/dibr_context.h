@@ -64,7 +64,7 @@ struct dibr_ctx {
   int args_zguard = 0;
   int plan_key[8] = {};   // what the plan below was made for (dibr_api.cu plan_band)
   dibr::BandPlan plan{};
-  int band_tables(const dibr_params *p);  // fills args.lut_h / lut_n, returns the guard width
+  int band_tables(const dibr_params *p);  // fills args.lut_h / frac, returns the guard width
 
   // batched launches (dibr_batch.cu)
   dibr::DevBuf batch_desc, batch_img, batch_depth;

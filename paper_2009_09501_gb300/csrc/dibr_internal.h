@@ -101,7 +101,7 @@ struct BandArgs {
   int *status;
   unsigned long long timeout_ns;
   int32_t lut_h[256];  // low 16 bits: hL[d], high 16 bits: hR[d] (signed)
-  int32_t lut_n[256];  // 510 * s_L(d): Fig. 3 shift numerator for the literal gather
+  uint32_t frac[8];    // bit d: s_L(d) is no whole number (the literal gather's samples left of column 0)
 };
 
 // Shared-memory layout of the band kernel (bytes from the dynamic smem base).
@@ -160,7 +160,7 @@ struct alignas(16) ImageDesc {
   uint32_t outputs;
   int32_t warp_mode, depth_src, out_mode, pad[3];
   int32_t lut_h[256];
-  int32_t lut_n[256];
+  uint32_t frac[8];
 };
 
 static_assert(sizeof(ImageDesc) % 16 == 0, "descriptors are read as an array");

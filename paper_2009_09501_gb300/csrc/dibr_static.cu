@@ -15,7 +15,7 @@
 #include "dibr_internal.h"
 
 namespace dibr {
-void shift_tables(const dibr_params *p, int32_t *lut_h, int32_t *lut_n);
+void shift_tables(const dibr_params *p, int32_t *lut_h, uint32_t *frac);
 }
 
 using namespace dibr;
@@ -28,7 +28,8 @@ constexpr int kStaticMaxDevices = 64;
 constexpr size_t kDescOff = 256;  // [group counters][status] ... [descriptors] [units]
 constexpr int kStatusWord = kMaxClasses;  // int index of the status word in the header
 constexpr size_t kUnitsOff = (kDescOff + sizeof(ImageDesc) * kStaticMaxImages + 255) / 256 * 256;
-constexpr size_t kStaticBytes = kUnitsOff + sizeof(int4) * kStaticMaxUnits;  // 267,008 bytes
+constexpr size_t kStaticBytes = kUnitsOff + sizeof(int4) * kStaticMaxUnits;
+static_assert(kStaticBytes == 208128, "the size that dibr.h states");
 
 // Device scratch shared by every call on a device (each GPU that loads the library holds
 // it until the process exits).  Host code must not use its name as an address: the
@@ -170,7 +171,7 @@ extern "C" dibr_status dibr_synthesize_batch_static(int n, const dibr_image *img
     dd.out_mode = out_mode_of(pp.outputs, dd.out, o.pitch);
     dd.warp_mode = pp.warp_mode;
     dd.depth_src = pp.depth_rule == DIBR_DEPTH_LUMA_BINOM5 ? DS_BINOM5 : DS_LUMA;
-    shift_tables(&pp, dd.lut_h, dd.lut_n);
+    shift_tables(&pp, dd.lut_h, dd.frac);
   }
   // every image of one fixed output set: the launches use that set's kernel instance
   uint32_t fixed = 0;
