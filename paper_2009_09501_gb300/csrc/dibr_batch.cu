@@ -31,8 +31,9 @@ void shift_tables(const dibr_params *p, int32_t *lut_h, uint32_t *frac);
 static int batch_zguard(const dibr_params *p, int n_params) {
   int g = 4;
   for (int i = 0; i < n_params; ++i) {
-    int32_t lh[256], ln[256];
-    shift_tables(&p[i], lh, ln);
+    int32_t lh[256];
+    uint32_t frac[8];
+    shift_tables(&p[i], lh, frac);
     g = std::max(g, zguard_of(lh));
   }
   return g;

@@ -127,8 +127,9 @@ extern "C" dibr_status dibr_synthesize_batch_static(int n, const dibr_image *img
   // the z-buffer guard every image fits in: the largest shift of their tables
   int zguard = 4;
   for (int i = 0; i < n_params; ++i) {
-    int32_t lh[256], ln[256];
-    shift_tables(&p[i], lh, ln);
+    int32_t lh[256];
+    uint32_t frac[8];
+    shift_tables(&p[i], lh, frac);
     const int g = zguard_of(lh);
     if (g > zguard) zguard = g;
   }
