@@ -454,9 +454,21 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     ia.block = p->inpaint_block;
     ia.nbx = (W + ia.block - 1) / ia.block;
     ia.nblocks = ia.nbx * ((H + ia.block - 1) / ia.block);
-    if ((s = ensure(inpaint_order, sizeof(int32_t) * (2 * static_cast<size_t>(ia.nblocks) + 3))) != DIBR_OK) return s;
+    const size_t words = 2 * static_cast<size_t>((H + 31) / 32) * W;
+    const uint8_t *had = inpaint_order.ptr;
+    const size_t had_bytes = inpaint_order.bytes;
+    if ((s = ensure(inpaint_order, sizeof(int32_t) * (kInpaintHeads + words + 2 * static_cast<size_t>(ia.nblocks)))) != DIBR_OK) return s;
+    if (inpaint_order.ptr != had || inpaint_order.bytes != had_bytes) {  // a new buffer: its counters start at 0
+      e = cudaMemsetAsync(inpaint_order.ptr, 0, sizeof(int32_t) * kInpaintHeads, stream);
+      if (e != cudaSuccess) {
+        inpaint_order.bytes = 0;  // (allocated and zeroed again by the next frame)
+        return cuda_fail(e, "inpainting scratch");
+      }
+    }
     ia.sms = num_sms;
-    ia.order = reinterpret_cast<int32_t *>(inpaint_order.ptr);
+    ia.heads = reinterpret_cast<int32_t *>(inpaint_order.ptr);
+    ia.planes = reinterpret_cast<uint32_t *>(ia.heads + kInpaintHeads);
+    ia.order = reinterpret_cast<int32_t *>(ia.planes + words);
     e = launch_inpaint(ia, stream);
     if (e != cudaSuccess) return cuda_fail(e, "inpainting launch");
     ++launches;

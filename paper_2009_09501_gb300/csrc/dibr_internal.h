@@ -378,6 +378,7 @@ inline void order_by_area(int n, const BatchShape *shape, int *order) {
   }
 }
 
+constexpr int kInpaintHeads = 16;
 // Arguments of the 2-D block inpainting (dibr_inpaint.cu): both views are repaired in
 // place; anaglyph and HSBS (either may be null) are rewritten where a view changed.
 struct InpaintArgs {
@@ -388,9 +389,11 @@ struct InpaintArgs {
   uint8_t *ana, *hsbs;    // row pitch out_pitch
   int64_t out_pitch;
   int32_t W, H, block, nbx, nblocks, sms;
-  int32_t *order;         // device scratch of 2 nblocks + 3 ints: the work items (2 block +
-                          // view) in processing order, the two fill counters of that order and
-                          // the next item to take (zeroed before the launch)
+  // device scratch
+  int32_t *heads;         // kInpaintHeads ints, 0 between launches: the two fill counters of the
+                          // order, the next item to take, the warps that are done
+  uint32_t *planes;       // 2 ceil(H / 32) W words: the views' damage, 32 rows of a column each
+  int32_t *order;         // 2 nblocks ints: the work items (2 block + view) in processing order
 };
 
 // Host launchers (dibr_band*.cu, dibr_xbf.cu, dibr_inpaint.cu).

@@ -140,6 +140,13 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+// 16 bytes from global to shared memory (both 16-byte aligned), asynchronous for this thread
+// until cp_async_wait_all.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Shared-memory accesses by 32-bit shared address.  They are volatile asm: the
 // compiler keeps them in program order with the barriers (also volatile asm).
 __device__ __forceinline__ uint32_t lds_u8(uint32_t a) {
