@@ -165,13 +165,19 @@ __device__ __forceinline__ int inpaint_block(const InpaintArgs &a, int item, uin
     // by row to cells, which never reach a piece that is still to be read.
     const uint8_t *const row0 = view + static_cast<int64_t>(by0 - 1) * a.pitch;
     const uint32_t *const piece = cell + kStride * kStride - kStride * 32;
-    for (int j = lane >> 3; j < bh + 2; j += 4) {
-      const uint8_t *const row = row0 + j * a.pitch, *const end = row + 3 * static_cast<int64_t>(W);
-      const uint8_t *const p = reinterpret_cast<const uint8_t *>(
-                                   reinterpret_cast<uintptr_t>(row + 3 * static_cast<int64_t>(bx0 - 1)) & ~uintptr_t(15)) +
-                               16 * (lane & 7);
-      const int y = by0 - 1 + j;
-      if (y >= 0 && y < H && p + 16 > row && p < end) cp_async16(smem_addr(piece) + 128 * j + 16 * (lane & 7), p);
+    {
+      const int64_t row_bytes = 3 * static_cast<int64_t>(W);
+      const int j0 = max(lane >> 3, by0 > 0 ? 0 : (lane >> 3) == 0 ? 4 : 0);  // (no row above the image)
+      const int j1 = min(bh + 2, H - by0 + 1);
+      const uint8_t *row = row0 + j0 * a.pitch;
+      uint32_t to = smem_addr(piece) + 128 * j0 + 16 * (lane & 7);
+      for (int j = j0; j < j1; j += 4) {
+        const uintptr_t at = reinterpret_cast<uintptr_t>(row + 3 * static_cast<int64_t>(bx0 - 1)) & ~uintptr_t(15);
+        const uint8_t *const p = reinterpret_cast<const uint8_t *>(at) + 16 * (lane & 7);
+        if (p + 16 > row && p < row + row_bytes) cp_async16(to, p);
+        row += 4 * a.pitch;
+        to += 4 * 128;
+      }
     }
     cp_async_wait_all();
     __syncwarp();
