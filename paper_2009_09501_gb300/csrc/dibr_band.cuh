@@ -1219,9 +1219,12 @@ __device__ __forceinline__ void init_barriers(const Shm &m, int nb) {
 template <int DS, bool FWD, uint32_t OUTS, bool RAG, bool TM, int ZP>
 __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_constant__ BandArgs a) {
   static_assert(!TM || (OUTS != 0 && DS == DS_BINOM5), "tensor memory only in the fixed-set binomial instances");
-  // The next launch on the stream may start its set-up while this one runs (programmatic
-  // dependent launch); it waits below for this one to complete before any global access.
-  griddep_launch_dependents();
+  // The next launch on the stream may start while this one runs (programmatic dependent
+  // launch); unless the host knows its buffers to be disjoint from those of all launches that
+  // may still run then, it waits for this one to complete before any global access.  A launch
+  // that itself waits lets the next one start only after that, so that these launches are
+  // those since the last one that waited.
+  if (a.overlap) griddep_launch_dependents();
   extern __shared__ __align__(128) uint8_t smem[];
   const Shm m = carve(smem, a.nb, a.srow, a.nch, a.nchz, blockDim.x >> 5, a.zguard, a.zp);
   fill_luts<FWD>(m, a.lut_h);
@@ -1231,7 +1234,10 @@ __global__ void __launch_bounds__(kMaxConsumers, 1) band_kernel(const __grid_con
   // or whose inputs this launch's outputs may overwrite) has completed -- unless the host
   // knows this launch touches none of that launch's buffers; then the wait moves to the
   // end, so that this launch still completes after the previous one
-  if (!a.overlap) griddep_wait();
+  if (!a.overlap) {
+    griddep_wait();
+    griddep_launch_dependents();
+  }
   const int nr = a.row1 - a.row0;
   const int ys = a.row0 + static_cast<int>(static_cast<int64_t>(blockIdx.x) * nr / a.grid);
   const int ye = a.row0 + static_cast<int>(static_cast<int64_t>(blockIdx.x + 1) * nr / a.grid);

@@ -72,14 +72,24 @@ struct dibr_ctx {
   size_t batch_pinned_bytes = 0;
   cudaEvent_t batch_copy_done = nullptr;   // the last descriptor upload has read the staging
 
-  // the buffers of the last single-frame launch (a band launch, or the inpainting launch
-  // after one), when it is the last work on a stream the context owns: the next band launch
-  // may overlap it if their buffers are disjoint
+  // The single-frame launches that may still run when the next one starts (prev_band: the last of
+  // them is the last work on a stream the context owns): the next band launch may overlap them if
+  // its buffers and theirs are disjoint.  A launch that waits for the work before it lets the
+  // next one start only then, so that it is the first of a new list; the 2-D fill's too.
   struct Span {
     uintptr_t lo = 0, hi = 0;
   };
+  struct Flight {
+    Span in, depth, out[dibr::O_COUNT];  // read: input, cross-bilateral depth
+    bool frame = false;                  // a band launch that is the whole of this frame:
+    dibr_image img;
+    dibr_params p;
+    dibr_outputs o;
+  };
+  static constexpr int kMaxFlights = 16;  // (a 17th kind of frame waits for the others)
   bool prev_band = false;
-  Span prev_in, prev_depth, prev_out[dibr::O_COUNT];  // read: input, cross-bilateral depth
+  int n_flights = 0;
+  Flight flights[kMaxFlights];
   int inpaint_half = 0;  // the half of inpaint_scratch the next 2-D fill frame uses
   int xbf_half = 0;      // the half of xbf_depth the next cross-bilateral frame uses
 
