@@ -41,7 +41,7 @@
 // z-buffer keeps target x at x + shift, with the row's shift (0..15) chosen so that every thread's
 // 16 targets start on a 16-byte boundary of the output row; only the two chunks cut by the row's
 // ends are stored by words and bytes.  That is the RAG template flag: a 4031 x 3023 photo with
-// tight rows 780 -> 107 us, 1366 x 768 side by side 29.6 -> 10.0 us (repacked by a strided copy
+// tight rows 780 -> 61 us (of it 107 -> 66 by one z-buffer row per view), 1366 x 768 side by side 29.6 -> 8.9 us (repacked by a strided copy
 // and stored by bytes before); aligned images keep instances without it.
 //
 // Instances: the requested outputs are read from the arguments, or fixed at compile time for

@@ -22,9 +22,9 @@
 // the side-by-side frame.  A rank pass turns the holes map into column words of 32 rows and
 // orders the items heavily damaged first; a persistent kernel takes them in that order.
 //
-// Bound by instruction issue while every SM has 32 warps, then by the latency of the last
-// items' steps.  A 4K frame with 8 % holes (12,340 items, 23 steps with visits each): the
-// kernel 71 us, 37 M warp instructions; the frame with its band launch 115 us.  When every
+// Bound by the integer pipe and issue while every SM has 32 warps, then by the latency of the
+// last items' steps.  A 4K frame with 8 % holes (11,732 items, 26 steps with visits each): the
+// kernel 71 us, 45 M warp instructions; the frame with its band launch 114 us.  When every
 // dirty pixel was visited one at a time, the flags were read from the map and the colours
 // from the view by each item, byte by byte, and all parts of a block shared one origin: 125
 // us, 89 M, 170 us.

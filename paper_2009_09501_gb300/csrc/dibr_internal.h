@@ -256,7 +256,8 @@ struct BandLimits {
 
 // The most CTAs per SM within the limits (128 registers per thread: the kernels' launch bound;
 // 2048 threads per SM), two z-buffer rows per view unless one leaves room for more CTAs (rows of
-// 3857 to 4096 pixels: two CTAs instead of one, a 4031 x 3023 frame 99 -> 66 us; 1080p: four instead of three, 10.3 -> 9.1), and the deepest ring.  Returns
+// 3857 to 4096 pixels: two CTAs instead of one, a 4031 x 3023
+// frame 99 -> 66 us; 1080p: four instead of three, 10.3 -> 9.1), and the deepest ring.  Returns
 // false if no plan fits.
 inline bool plan_smem(BandPlan &p, const BandLimits &lim, int nc, int srow, int nch, int nchz, int zguard, int min_nb) {
   const int max_nb = lim.ring_slots <= 0 ? kMaxRing : lim.ring_slots < min_nb ? min_nb : lim.ring_slots < kMaxRing ? lim.ring_slots : kMaxRing;
