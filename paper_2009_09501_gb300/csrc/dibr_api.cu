@@ -346,8 +346,8 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     for (int k = 0; k < n_flights; ++k) {
       const Flight &f = flights[k];
       if (meets(cur_depth, f.in) || meets(cur_depth, f.depth)) after = false;
-      for (int i = 0; i < O_COUNT; ++i)
-        if (f.out[i].hi && (meets(xin, f.out[i]) || meets(cur_depth, f.out[i]))) after = false;
+      for (int i = 0; i < f.n_out; ++i)
+        if (meets(xin, f.out[i]) || meets(cur_depth, f.out[i])) after = false;
     }
     cudaError_t e = launch_xbf(in, pitch, W, H, p->xbf_radius, p->xbf_sigma_s, p->xbf_sigma_r, dd, dp, stream,
                                after);
@@ -407,14 +407,14 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   // its exit waits for it.  (The same frame again, a repeat of one in flight, writes the bytes
   // that one writes.)
   Span cur_in = span(in, pitch, H, 3 * static_cast<int64_t>(W)), cur_out[O_COUNT];
-  for (int i = 0; i < O_COUNT; ++i)
-    cur_out[i] = (a.outputs & kOutBits[i]) && a.out[i]
-                     ? span(a.out[i], is_map_output(i) ? a.depth_pitch : a.out_pitch, H,
-                            is_map_output(i) ? static_cast<int64_t>(W) : 3 * static_cast<int64_t>(W))
-                     : Span{};
+  int n_out = 0;
   bool disjoint = may_overlap && !scratch, in_place = false;
-  for (int i = 0; i < O_COUNT; ++i)
-    if (cur_out[i].hi && meets(cur_in, cur_out[i])) in_place = true;
+  for (int i = 0; i < O_COUNT; ++i) {
+    if (!(a.outputs & kOutBits[i]) || !a.out[i]) continue;
+    cur_out[n_out] = span(a.out[i], is_map_output(i) ? a.depth_pitch : a.out_pitch, H,
+                          is_map_output(i) ? static_cast<int64_t>(W) : 3 * static_cast<int64_t>(W));
+    if (meets(cur_in, cur_out[n_out++])) in_place = true;
+  }
   int again = -1;
   for (int k = 0; k < n_flights && disjoint; ++k) {
     const Flight &f = flights[k];
@@ -423,12 +423,12 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
       again = k;
       continue;
     }
-    for (int i = 0; i < O_COUNT; ++i) {
-      if (f.out[i].hi && meets(cur_in, f.out[i])) disjoint = false;  // reads what it wrote
-      if (!cur_out[i].hi) continue;
+    for (int j = 0; j < f.n_out; ++j)
+      if (meets(cur_in, f.out[j])) disjoint = false;  // reads what it wrote
+    for (int i = 0; i < n_out; ++i) {
       if (meets(cur_out[i], f.in) || meets(cur_out[i], f.depth)) disjoint = false;  // writes what it read
-      for (int j = 0; j < O_COUNT; ++j)
-        if (f.out[j].hi && meets(cur_out[i], f.out[j])) disjoint = false;  // writes what it wrote
+      for (int j = 0; j < f.n_out; ++j)
+        if (meets(cur_out[i], f.out[j])) disjoint = false;  // writes what it wrote
     }
   }
   if (again < 0 && n_flights == kMaxFlights) disjoint = false;
@@ -460,7 +460,8 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     Flight &f = flights[n_flights++];
     f.in = cur_in;
     f.depth = cur_depth;
-    for (int i = 0; i < O_COUNT; ++i) f.out[i] = cur_out[i];
+    f.n_out = n_out;
+    for (int i = 0; i < n_out; ++i) f.out[i] = cur_out[i];
     f.frame = !scratch;
     f.img = *img;
     f.p = *p;
@@ -505,7 +506,8 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     n_flights = 1;
     Flight &f = flights[0];
     f = Flight{};
-    for (int i = 0; i < O_COUNT; ++i) f.out[i] = cur_out[i];
+    f.n_out = n_out;
+    for (int i = 0; i < n_out; ++i) f.out[i] = cur_out[i];
   }
   return DIBR_OK;
 }

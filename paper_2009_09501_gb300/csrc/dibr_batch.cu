@@ -66,11 +66,22 @@ void dibr_ctx::release_batch_buffers() {
 }
 
 // All buffers in device memory.  Images large enough to fill the GPU on their own (at
-// least kOwnLaunchRows rows per CTA slot of their launch plan; e.g. 4K and 8K frames) get a
-// band launch each, back to back, overlapping one another when their buffers are disjoint;
-// measured, that beats the persistent launch for them.  The others (e.g. 1080p, 720p) share
-// the grouped persistent launches, which beat per-image launches for them.
+// least kOwnLaunchRows rows per CTA slot of a plan with two z-buffer rows per view; e.g. 1440p,
+// 4K and 8K frames) get a band launch each, back to back, overlapping one another when their
+// buffers are disjoint; measured, that beats the persistent launch for them.  The others (e.g.
+// 1080p, 720p) share the grouped persistent launches, which beat per-image launches for them.
+// (With the slots of the one-row plans, 1440p frames would share: 2560 x 1440 and two larger
+// frames 172 us, 70 so -- the shared launch's descriptors take an upload.)
 constexpr int kOwnLaunchRows = 4;
+
+// CTAs per SM of the two-row plan; 0: does not fit.
+static int two_row_ctas(const BatchShape &s, const BatchLimits &lim) {
+  const int nc = block_of(s), min_nb = 4;
+  const int tot = band_smem_layout(min_nb, slot_bytes(s.width, s.aligned), chunks_of(s.width), s.nchz, nc / 32, lim.zguard, 2).total;
+  if (tot > lim.band.max_smem) return 0;
+  const int per = std::min(lim.band.smem_per_sm / (tot + 1024), std::min(65536 / (nc * 128), 2048 / nc));
+  return lim.band.ctas_per_sm > 0 ? std::min(per, lim.band.ctas_per_sm) : per;
+}
 
 dibr_status dibr_ctx::enqueue_batch_device(int n, const dibr_image *imgs, const dibr_params *p, int n_params,
                                            const dibr_outputs *outs) {
@@ -82,7 +93,8 @@ dibr_status dibr_ctx::enqueue_batch_device(int n, const dibr_image *imgs, const 
     int cl = 0;
     BatchClass c[1];
     const bool fits = plan_batch_classes(1, &shape, lim, &cl, c) == 1;
-    const int64_t slots = static_cast<int64_t>(num_sms) * (fits ? c[0].per : 1);
+    const int two = fits ? two_row_ctas(shape, lim) : 0;
+    const int64_t slots = static_cast<int64_t>(num_sms) * (two ? two : fits ? c[0].per : 1);
     bool big = fits && tuning.rows_per_unit == 0 && imgs[i].height >= kOwnLaunchRows * slots;
     const auto t = class_tune.find(block_of(shape));
     if (fits && tuning.rows_per_unit == 0 && t != class_tune.end() && t->second.own >= 0) big = t->second.own == 1;

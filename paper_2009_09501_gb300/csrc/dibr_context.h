@@ -80,13 +80,14 @@ struct dibr_ctx {
     uintptr_t lo = 0, hi = 0;
   };
   struct Flight {
-    Span in, depth, out[dibr::O_COUNT];  // read: input, cross-bilateral depth
+    Span in, depth, out[dibr::O_COUNT];  // read: input, cross-bilateral depth; n_out written
+    int n_out = 0;
     bool frame = false;                  // a band launch that is the whole of this frame:
     dibr_image img;
     dibr_params p;
     dibr_outputs o;
   };
-  static constexpr int kMaxFlights = 16;  // (a 17th kind of frame waits for the others)
+  static constexpr int kMaxFlights = 64;  // (a 65th kind of frame in a row waits for the others)
   bool prev_band = false;
   int n_flights = 0;
   Flight flights[kMaxFlights];
