@@ -806,6 +806,9 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
       f = make_uint4(~d.x, ~d.y, ~d.z, ~d.w);
     }
     if (want_depth && active && !depth_bytes(y)) store16(a.out[O_DEPTH] + static_cast<int64_t>(y) * a.depth_pitch + x0, make_uint4(~f.x, ~f.y, ~f.z, ~f.w), npx);
+    // (the lanes' reads of the row before are done, and rows_ab orders this store before the next
+    // reads: B reads other lanes' bytes, by loads that the compiler may move across plain stores)
+    __syncwarp();
     if (wfull || own_chunk) *reinterpret_cast<uint4 *>(m.drow + x0) = f;
   };
 
@@ -1163,6 +1166,7 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
   // for a second CTA on the SM) right after its own row's.
   auto rows_ab = [&](int y) {
     phase_a(y);
+    __syncwarp();  // the warp's part of the depth row is written
     phase_b(y);
     arrive_b(y);
   };
