@@ -164,21 +164,16 @@ __device__ __forceinline__ int inpaint_block(const InpaintArgs &a, int item, uin
     // rows in flight at once, into rows of 128 bytes at the end of the cells' space; then row
     // by row to cells, which never reach a piece that is still to be read.
     const uint8_t *const row0 = view + static_cast<int64_t>(by0 - 1) * a.pitch;
-    const uint32_t *const piece = cell + kStride * kStride - kStride * 32;
-    {
-      const int64_t row_bytes = 3 * static_cast<int64_t>(W);
-      const int j0 = max(lane >> 3, by0 > 0 ? 0 : (lane >> 3) == 0 ? 4 : 0);  // (no row above the image)
-      const int j1 = min(bh + 2, H - by0 + 1);
-      const uint8_t *row = row0 + j0 * a.pitch;
-      uint32_t to = smem_addr(piece) + 128 * j0 + 16 * (lane & 7);
-      for (int j = j0; j < j1; j += 4) {
-        const uintptr_t at = reinterpret_cast<uintptr_t>(row + 3 * static_cast<int64_t>(bx0 - 1)) & ~uintptr_t(15);
-        const uint8_t *const p = reinterpret_cast<const uint8_t *>(at) + 16 * (lane & 7);
-        if (p + 16 > row && p < row + row_bytes) cp_async16(to, p);
-        row += 4 * a.pitch;
-        to += 4 * 128;
-      }
-    }
+    uint32_t *const piece = cell + kStride * kStride - kStride * 32;
+    // (a unit that reaches past the view's first or last byte is fetched byte by byte: nothing
+    // outside the view is read)
+    frame_units(
+        view, a.pitch, W, H, bx0, by0, bh, lane,
+        [&](int j, const uint8_t *u) { cp_async16(smem_addr(piece) + 128 * j + 16 * (lane & 7), u); },
+        [&](int j, const uint8_t *u, int b0, int b1) {
+          uint8_t *const to = reinterpret_cast<uint8_t *>(piece) + 128 * j + 16 * (lane & 7);
+          for (int b = b0; b < b1; ++b) to[b] = u[b];
+        });
     cp_async_wait_all();
     __syncwarp();
     const uint32_t s0 = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(row0)) + 3u * (bx0 - 1);

@@ -397,6 +397,30 @@ struct InpaintArgs {
   int32_t *order;         // 2 nblocks ints: the work items (2 block + view) in processing order
 };
 
+// The 16-byte units that hold the frame of an inpainting block at (bx0, by0), bh rows high: its
+// rows and columns and one more on every side, so at most 34 x 3 bytes of a row, at any offset: 8
+// units.  One lane's share of them (unit lane % 8 of every fourth frame row from lane / 8 on;
+// frame row j is row by0 - 1 + j): whole(j, u) for the unit at u, part(j, u, b0, b1) for one that
+// reaches past the view's memory, of which bytes b0 .. b1 - 1 are the view's.  Only rows next to
+// the view's first and last byte can have such units: `inside` rules them out for all others.
+template <class Whole, class Part>
+__host__ __device__ inline void frame_units(const uint8_t *view, int64_t pitch, int W, int H, int bx0, int by0, int bh,
+                                            int lane, Whole whole, Part part) {
+  const int64_t row_bytes = 3 * static_cast<int64_t>(W);
+  const uint8_t *const end = view + (H - 1) * pitch + row_bytes;
+  const int first = by0 > 0 ? by0 - 1 : 0, last = by0 + bh < H ? by0 + bh : H - 1;
+  const bool inside = first * pitch >= 15 && (H - 1 - last) * pitch >= 15;
+  const int j0 = by0 == 0 && (lane >> 3) == 0 ? 4 : lane >> 3;  // (no row above the image)
+  const uint8_t *row = view + (by0 - 1 + j0) * pitch;
+  for (int j = j0; j <= last - by0 + 1; j += 4, row += 4 * pitch) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(row + 3 * static_cast<int64_t>(bx0 - 1)) & ~static_cast<uintptr_t>(15);
+    const uint8_t *const u = reinterpret_cast<const uint8_t *>(at) + 16 * (lane & 7);
+    if (u + 16 <= row || u >= row + row_bytes) continue;
+    if (inside || (u >= view && u + 16 <= end)) whole(j, u);
+    else part(j, u, u < view ? static_cast<int>(view - u) : 0, u + 16 > end ? static_cast<int>(end - u) : 16);
+  }
+}
+
 // Host launchers (dibr_band*.cu, dibr_xbf.cu, dibr_inpaint.cu).
 cudaError_t launch_band_ragged(const BandArgs &a, int smem_bytes, cudaStream_t st);
 cudaError_t launch_band_any(const BandArgs &a, int smem_bytes, cudaStream_t st);
