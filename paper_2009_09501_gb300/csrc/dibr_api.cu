@@ -486,19 +486,23 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     const uint8_t *had = inpaint_order.ptr;
     const size_t had_bytes = inpaint_order.bytes;
     if ((s = ensure(inpaint_order, sizeof(int32_t) * (kInpaintHeads + words + 2 * static_cast<size_t>(ia.nblocks)))) != DIBR_OK) return s;
-    if (inpaint_order.ptr != had || inpaint_order.bytes != had_bytes) {  // a new buffer: its counters start at 0
-      e = cudaMemsetAsync(inpaint_order.ptr, 0, sizeof(int32_t) * kInpaintHeads, stream);
-      if (e != cudaSuccess) {
-        inpaint_order.bytes = 0;  // (allocated and zeroed again by the next frame)
-        return cuda_fail(e, "inpainting scratch");
-      }
-    }
+    if (inpaint_order.ptr != had || inpaint_order.bytes != had_bytes) inpaint_heads_zero = false;
+    // The counters are zeroed here unless the frame before left them at 0, which the end of its
+    // inpainting does: not in a new buffer, not after a launch that failed between the two, and
+    // in a capture always (what it records may run after any other frame; it zeroes nothing now).
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(stream, &cap);
+    const bool eager = e == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    if (e == cudaSuccess && !(eager && inpaint_heads_zero)) e = cudaMemsetAsync(inpaint_order.ptr, 0, sizeof(int32_t) * kInpaintHeads, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "inpainting scratch");
     ia.sms = num_sms;
     ia.heads = reinterpret_cast<int32_t *>(inpaint_order.ptr);
     ia.planes = reinterpret_cast<uint32_t *>(ia.heads + kInpaintHeads);
     ia.order = reinterpret_cast<int32_t *>(ia.planes + words);
+    if (eager) inpaint_heads_zero = false;
     e = launch_inpaint(ia, stream);
     if (e != cudaSuccess) return cuda_fail(e, "inpainting launch");
+    if (eager) inpaint_heads_zero = true;
     ++launches;
     // the inpainting reads and writes the band launch's outputs (views, holes map,
     // anaglyph, side-by-side) and nothing else the next frame's band launch could touch

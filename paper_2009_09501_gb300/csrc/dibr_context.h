@@ -92,6 +92,7 @@ struct dibr_ctx {
   int n_flights = 0;
   Flight flights[kMaxFlights];
   int inpaint_half = 0;  // the half of inpaint_scratch the next 2-D fill frame uses
+  bool inpaint_heads_zero = false;  // the counters in inpaint_order are 0 when the work enqueued so far is done
   int xbf_half = 0;      // the half of xbf_depth the next cross-bilateral frame uses
 
   // blocking calls with host buffers: copies and kernels of row bands overlap

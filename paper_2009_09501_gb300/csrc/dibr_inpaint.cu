@@ -117,7 +117,8 @@ __global__ void __launch_bounds__(32 * kRankWarps) inpaint_rank_kernel(const __g
   __syncthreads();
   if (place) {
     pos += base[heavy ? 0 : 1];
-    a.order[heavy ? pos : 2 * a.nblocks - 1 - pos] = 2 * unit + lane;
+    // (inside the order whatever the counters held)
+    if (static_cast<uint32_t>(pos) < 2u * a.nblocks) a.order[heavy ? pos : 2 * a.nblocks - 1 - pos] = 2 * unit + lane;
   }
 }
 
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(32 * kWarps, kCtas) inpaint_kernel(const __gri
   // buffers are disjoint).
   griddep_launch_dependents();
   // the order holds nh heavy items at its front and nl others at its back
-  const int items = 2 * a.nblocks, nh = a.heads[0], n = nh + a.heads[1];
+  const int items = 2 * a.nblocks, nh = min(a.heads[0], items), n = min(nh + a.heads[1], items);
   const bool leader = (threadIdx.x & 31) == 0;
   // A warp's first item is its own number in the grid, CTA first: consecutive CTAs start on
   // different SMs, so the heavy items spread over all of them (first come, first served gave
@@ -431,8 +432,7 @@ __global__ void __launch_bounds__(32 * kWarps, kCtas) inpaint_kernel(const __gri
 
 }  // namespace
 
-// The counters of InpaintArgs::heads are 0 here: zeroed with the allocation and left so by each
-// launch.
+// The counters of InpaintArgs::heads are 0 here (the caller's part), and again after both launches.
 cudaError_t launch_inpaint(const InpaintArgs &a, cudaStream_t st) {
   if (a.nblocks <= 0) return cudaSuccess;
   const int tiles = a.block == kMaxBlock ? 0 : ((a.W + 31) / 32) * ((a.H + 31) / 32);

@@ -391,8 +391,8 @@ struct InpaintArgs {
   int64_t out_pitch;
   int32_t W, H, block, nbx, nblocks, sms;
   // device scratch
-  int32_t *heads;         // kInpaintHeads ints, 0 between launches: the two fill counters of the
-                          // order, the next item to take, the warps that are done
+  int32_t *heads;         // kInpaintHeads ints, 0 before and after a frame's two launches: the two
+                          // fill counters of the order, the next item to take, the warps that are done
   uint32_t *planes;       // 2 ceil(H / 32) W words: the views' damage, 32 rows of a column each
   int32_t *order;         // 2 nblocks ints: the work items (2 block + view) in processing order
 };
