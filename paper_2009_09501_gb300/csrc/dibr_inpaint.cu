@@ -422,7 +422,8 @@ __global__ void __launch_bounds__(32 * kWarps, kCtas) inpaint_kernel(const __gri
   while (i < n) {
     const int item = a.order[i < nh ? i : items - n + i];
     const int taken = inpaint_block(a, item, cells[threadIdx.x >> 5], recip);
-    i = warps + __shfl_sync(0xffffffffu, taken, 0);  // (and the cells are free)
+    i = warps + __shfl_sync(0xffffffffu, taken, 0);
+    __syncwarp();  // every lane has read its cells: they are free for the next item's pieces
   }
   if (leader && atomicAdd(&a.heads[3], 1) == warps - 1) {
 #pragma unroll
