@@ -174,20 +174,31 @@ void shift_tables(const dibr_params *p, int32_t *lut_h, uint32_t *frac) {
 }  // namespace dibr
 
 // ---------------------------------------------------------------- launch planning
-static PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+// Driver entry points, looked up once.  The stream's state is asked through the driver: every
+// enqueued frame asks twice, and the runtime's calls of the same name take 0.1 us more each (a
+// 640x480 frame every 4.0 us is the host's).
+struct Driver {
+  PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  PFN_cuStreamIsCapturing_v10000 is_capturing = nullptr;
+  PFN_cuStreamQuery_v2000 query = nullptr;
+};
+static const Driver &driver() {
+  static Driver d;
   static std::once_flag once;
   std::call_once(once, [] {
-    void *f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
-    else
+    auto find = [](const char *name, unsigned version) -> void * {
+      void *f = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      if (cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+        return f;
       cudaGetLastError();
+      return nullptr;
+    };
+    d.encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(find("cuTensorMapEncodeTiled", 12000));
+    d.is_capturing = reinterpret_cast<PFN_cuStreamIsCapturing_v10000>(find("cuStreamIsCapturing", 10000));
+    d.query = reinterpret_cast<PFN_cuStreamQuery_v2000>(find("cuStreamQuery", 2000));
   });
-  return fn;
+  return d;
 }
 
 int dibr_ctx::band_tables(const dibr_params *p) {
@@ -274,7 +285,7 @@ dibr_status dibr_ctx::plan_band(int W, int H, int depth_src, const uint8_t *in, 
 
 dibr_status dibr_ctx::encode_input(BandArgs &a, const uint8_t *dev_rgb, int64_t pitch) {
   if (a.load_mode == LM_BULK) return DIBR_OK;  // no tensor map needed
-  auto enc = get_encoder();
+  const auto enc = driver().encode;
   if (!enc) {
     set_error("cuTensorMapEncodeTiled is unavailable");
     return DIBR_E_CUDA;
@@ -311,8 +322,16 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   const uint8_t *in = img->rgb;
   const int64_t pitch = img->pitch;
   // this launch may overlap the previous one (see below) only if that was the last work
-  // on a stream the context owns
-  const bool may_overlap = owns_stream && prev_band;
+  // on a stream the context owns, and neither is only recorded by a capture: a recorded launch
+  // runs some other time, behind work this context does not know
+  cudaError_t e;
+  CUstreamCaptureStatus cap = CU_STREAM_CAPTURE_STATUS_NONE;
+  if (driver().is_capturing(stream, &cap) != CUDA_SUCCESS) {
+    set_error("the context's stream cannot be used");
+    return DIBR_E_CUDA;
+  }
+  const bool eager = cap == CU_STREAM_CAPTURE_STATUS_NONE;
+  const bool may_overlap = owns_stream && prev_band && eager;
   prev_band = false;
   auto span = [](const uint8_t *ptr, int64_t row_pitch, int rows, int64_t row_bytes) {
     Span sp;
@@ -349,8 +368,7 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
       for (int i = 0; i < f.n_out; ++i)
         if (meets(xin, f.out[i]) || meets(cur_depth, f.out[i])) after = false;
     }
-    cudaError_t e = launch_xbf(in, pitch, W, H, p->xbf_radius, p->xbf_sigma_s, p->xbf_sigma_r, dd, dp, stream,
-                               after);
+    e = launch_xbf(in, pitch, W, H, p->xbf_radius, p->xbf_sigma_s, p->xbf_sigma_r, dd, dp, stream, after);
     if (e != cudaSuccess) return cuda_fail(e, "cross-bilateral launch");
     ++launches;
     a.depth_in = dd;
@@ -444,18 +462,16 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   // two and with one; 1440p 91, 65 and 75).
   const int fif = tuning.frames_in_flight > 0 ? tuning.frames_in_flight : kFramesInFlight;
   const int full_grid = a.grid;
-  if (disjoint && !inpaint && fif > 1 && per_sm >= 2 && cudaStreamQuery(stream) == cudaErrorNotReady) {
-    if (cudaPeekAtLastError() == cudaErrorNotReady) cudaGetLastError();  // (not an error)
+  if (disjoint && !inpaint && fif > 1 && per_sm >= 2 && driver().query(stream) == CUDA_ERROR_NOT_READY)
     a.grid = std::max(1, std::min(a.grid, (num_sms * per_sm + fif - 1) / fif));
-  }
   if (inpaint) a.grid = std::min(a.grid, 2 * num_sms);
-  cudaError_t e = launch_band(a, smem, stream);
+  e = launch_band(a, smem, stream);
   a.overlap = 0;
   a.grid = full_grid;
   if (e != cudaSuccess) return cuda_fail(e, "band kernel launch");
   ++launches;
   if (!disjoint) n_flights = 0;
-  if (!inpaint) prev_band = true;
+  if (!inpaint) prev_band = eager;
   if (!inpaint && (again < 0 || !disjoint)) {
     Flight &f = flights[n_flights++];
     f.in = cur_in;
@@ -490,11 +506,9 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     // The counters are zeroed here unless the frame before left them at 0, which the end of its
     // inpainting does: not in a new buffer, not after a launch that failed between the two, and
     // in a capture always (what it records may run after any other frame; it zeroes nothing now).
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    e = cudaStreamIsCapturing(stream, &cap);
-    const bool eager = e == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-    if (e == cudaSuccess && !(eager && inpaint_heads_zero)) e = cudaMemsetAsync(inpaint_order.ptr, 0, sizeof(int32_t) * kInpaintHeads, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "inpainting scratch");
+    if (!(eager && inpaint_heads_zero) &&
+        (e = cudaMemsetAsync(inpaint_order.ptr, 0, sizeof(int32_t) * kInpaintHeads, stream)) != cudaSuccess)
+      return cuda_fail(e, "inpainting scratch");
     ia.sms = num_sms;
     ia.heads = reinterpret_cast<int32_t *>(inpaint_order.ptr);
     ia.planes = reinterpret_cast<uint32_t *>(ia.heads + kInpaintHeads);
@@ -506,7 +520,7 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     ++launches;
     // the inpainting reads and writes the band launch's outputs (views, holes map,
     // anaglyph, side-by-side) and nothing else the next frame's band launch could touch
-    prev_band = true;
+    prev_band = eager;
     n_flights = 1;
     Flight &f = flights[0];
     f = Flight{};
@@ -612,6 +626,7 @@ dibr_status dibr_create(const dibr_config *cfg_in, dibr_ctx **out) {
   if (cudaGetDeviceProperties(&prop, cfg.device) != cudaSuccess) return DIBR_E_CUDA;
   if (!(prop.major == 10 && prop.minor == 3)) return DIBR_E_CUDA;  // built for sm_103a only
   if (cudaSetDevice(cfg.device) != cudaSuccess) return DIBR_E_CUDA;
+  if (!driver().is_capturing || !driver().query) return DIBR_E_CUDA;
   dibr_ctx *c = new dibr_ctx();
   c->device = cfg.device;
   c->num_sms = prop.multiProcessorCount;

@@ -125,8 +125,21 @@ cudaError_t cudaGetDeviceProperties(cudaDeviceProp *p, int) {
   p->sharedMemPerMultiprocessor = 233472;
   return cudaSuccess;
 }
-cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **f, unsigned, unsigned long long, cudaDriverEntryPointQueryResult *) {
-  return *f = nullptr, cudaErrorUnknown;
+CUresult fake_is_capturing(CUstream, CUstreamCaptureStatus *s) {
+  std::lock_guard<std::mutex> g(mu);
+  *s = capturing ? CU_STREAM_CAPTURE_STATUS_ACTIVE : CU_STREAM_CAPTURE_STATUS_NONE;
+  return CUDA_SUCCESS;
+}
+CUresult fake_query(CUstream) {
+  std::lock_guard<std::mutex> g(mu);
+  if (capturing) text += "query while capturing\n";
+  return capturing ? CUDA_ERROR_STREAM_CAPTURE_UNSUPPORTED : busy ? CUDA_ERROR_NOT_READY : CUDA_SUCCESS;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char *name, void **f, unsigned, unsigned long long, cudaDriverEntryPointQueryResult *q) {
+  const std::string n = name;
+  *f = n == "cuStreamIsCapturing" ? reinterpret_cast<void *>(fake_is_capturing) : n == "cuStreamQuery" ? reinterpret_cast<void *>(fake_query) : nullptr;
+  *q = *f ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+  return cudaSuccess;
 }
 const char *cudaGetErrorString(cudaError_t) { return "a fake error"; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
@@ -142,15 +155,15 @@ cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return std::free(p), cudaSucc
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return handle(s); }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return note("cudaStreamSynchronize", "sync"); }
-cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) {
-  std::lock_guard<std::mutex> g(mu);
-  *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+cudaError_t cudaStreamIsCapturing(cudaStream_t st, cudaStreamCaptureStatus *s) {
+  CUstreamCaptureStatus c;
+  fake_is_capturing(st, &c);
+  *s = static_cast<cudaStreamCaptureStatus>(c);
   return cudaSuccess;
 }
-cudaError_t cudaStreamQuery(cudaStream_t) {
-  std::lock_guard<std::mutex> g(mu);
-  if (capturing) text += "query while capturing\n";
-  return capturing ? cudaErrorStreamCaptureUnsupported : busy ? cudaErrorNotReady : cudaSuccess;
+cudaError_t cudaStreamQuery(cudaStream_t st) {
+  const CUresult r = fake_query(st);
+  return r == CUDA_ERROR_NOT_READY ? cudaErrorNotReady : r == CUDA_SUCCESS ? cudaSuccess : cudaErrorStreamCaptureUnsupported;
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) { return note("cudaStreamWaitEvent", "wait" + id(s) + id(e)); }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return handle(e); }
