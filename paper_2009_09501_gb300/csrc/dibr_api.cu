@@ -457,14 +457,14 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   // one after the other across every SM.  Both CTAs of an SM must fit at once.  Not with the
   // 2-D fill: its launches follow this one and nothing of another frame runs beside it, so a
   // share of the SMs only made it longer (4K frames back to back 334 us, 114 on every SM).
-  // Two CTAs an SM are enough there: more leave a CTA two rows beside the five its first row
+  // Two CTAs an SM are enough there, unless the tuning says how many: more leave a CTA two rows beside the five its first row
   // needs, and the launches behind it no room to be ready in (1080p 71 us with four, 49 with
   // two and with one; 1440p 91, 65 and 75).
   const int fif = tuning.frames_in_flight > 0 ? tuning.frames_in_flight : kFramesInFlight;
   const int full_grid = a.grid;
   if (disjoint && !inpaint && fif > 1 && per_sm >= 2 && driver().query(stream) == CUDA_ERROR_NOT_READY)
     a.grid = std::max(1, std::min(a.grid, (num_sms * per_sm + fif - 1) / fif));
-  if (inpaint) a.grid = std::min(a.grid, 2 * num_sms);
+  if (inpaint && tuning.ctas_per_sm == 0) a.grid = std::min(a.grid, 2 * num_sms);
   e = launch_band(a, smem, stream);
   a.overlap = 0;
   a.grid = full_grid;

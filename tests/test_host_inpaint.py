@@ -1,5 +1,5 @@
-"""The 2-D fill's counters between frames, by the calls the host makes (a recording CUDA runtime,
-no GPU): zeroed before every frame that does not follow a frame that left them at 0.  CPU only."""
+"""The 2-D fill by the calls the host makes (a recording CUDA runtime, no GPU): its counters are
+zeroed before every frame that does not follow a frame that left them at 0; its grid.  CPU only."""
 import pytest
 
 import fakecuda
@@ -64,3 +64,15 @@ def test_a_captured_frame_carries_its_own_memset(fake, ctx):
     fake.fake_state(0, 0)
     assert _frame(fake, ctx) == (D.DIBR_OK, ZEROED)  # nothing captured has run
     assert _frame(fake, ctx) == (D.DIBR_OK, WHOLE)
+
+
+# The 2-D fill's band launch: two CTAs an SM at most (152 SMs), or as many as the tuning asks for
+# and the plan allows (1080 rows of 1920 columns: four an SM).
+@pytest.mark.parametrize("ctas,grid", [(0, 304), (1, 152), (2, 304), (3, 456), (4, 608), (8, 608)])
+def test_tuned_ctas_per_sm(fake, ctx, ctas, grid):
+    assert fake.dibr_set_tuning(ctx, D.dibr_tuning(ctas_per_sm=ctas)) == D.DIBR_OK
+    fake.take()
+    p = D.make_params(outputs=NAMES, hole_fill=D.DIBR_FILL_INPAINT2D)
+    assert fake.dibr_enqueue_image(ctx, fakecuda.image(1920, 1080), p, fakecuda.outputs(NAMES, 1920)) == D.DIBR_OK
+    band = [w for w in fake.take() if w[:2] == ["launch", "band_kernel"]]
+    assert [int(w[2]) for w in band] == [grid]
