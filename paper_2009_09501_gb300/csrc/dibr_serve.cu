@@ -239,7 +239,9 @@ static void scheduler_loop(ServeState *st) {
     for (size_t f = 0; f < n && status == DIBR_OK;) {
       const size_t bytes = static_cast<size_t>(imgs[f].pitch) * imgs[f].height;
       const int H = imgs[f].height;
-      const bool rows = prms[f].depth_rule != DIBR_DEPTH_LUMA_XBF;  // (its depth pass takes the whole frame)
+      // a launch of the frame's own rows: not with the cross-bilateral depth, whose pass takes the whole
+      // frame, nor where the tuning sets the rows of a batched launch's units
+      const bool rows = prms[f].depth_rule != DIBR_DEPTH_LUMA_XBF && st->gpu->tuning.rows_per_unit == 0;
       const int bands = rows && others < 2 ? std::max(1, std::min(static_cast<int>(std::min<size_t>(kMaxParts, bytes / kPartBytes)), H / 8)) : 1;
       if (bands > 1) {
         auto row = [&](int j) { return static_cast<int>(static_cast<int64_t>(j) * H / bands); };
