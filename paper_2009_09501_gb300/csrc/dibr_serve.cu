@@ -236,13 +236,16 @@ static void scheduler_loop(ServeState *st) {
     // frames or more in flight their copies fill the link already, and bands only add copies (4K
     // frames streamed three at a time: 2,266 frames/s in bands, 2,370 whole).
     const size_t n = imgs.size();
+    // a launch of the frame's own rows: not with the cross-bilateral depth, whose pass takes the whole
+    // frame, nor where the tuning sets the rows of a batched launch's units
+    auto own_rows = [&](size_t f) { return prms[f].depth_rule != DIBR_DEPTH_LUMA_XBF && st->gpu->tuning.rows_per_unit == 0; };
+    auto bytes_of = [&](size_t f) { return static_cast<size_t>(imgs[f].pitch) * imgs[f].height; };
+    auto bands_of = [&](size_t f) {  // (of a large frame: more than one)
+      if (!own_rows(f)) return 1;
+      return std::max(1, std::min(static_cast<int>(std::min<size_t>(kMaxParts, bytes_of(f) / kPartBytes)), imgs[f].height / 8));
+    };
     for (size_t f = 0; f < n && status == DIBR_OK;) {
-      const size_t bytes = static_cast<size_t>(imgs[f].pitch) * imgs[f].height;
-      const int H = imgs[f].height;
-      // a launch of the frame's own rows: not with the cross-bilateral depth, whose pass takes the whole
-      // frame, nor where the tuning sets the rows of a batched launch's units
-      const bool rows = prms[f].depth_rule != DIBR_DEPTH_LUMA_XBF && st->gpu->tuning.rows_per_unit == 0;
-      const int bands = rows && others < 2 ? std::max(1, std::min(static_cast<int>(std::min<size_t>(kMaxParts, bytes / kPartBytes)), H / 8)) : 1;
+      const int H = imgs[f].height, bands = others < 2 ? bands_of(f) : 1;
       if (bands > 1) {
         auto row = [&](int j) { return static_cast<int>(static_cast<int64_t>(j) * H / bands); };
         upload(f, 0, row(1));
@@ -258,11 +261,11 @@ static void scheduler_loop(ServeState *st) {
         continue;
       }
       size_t end = f, sum = 0;
-      while (end < n && (end == f || sum < kPartBytes)) sum += static_cast<size_t>(imgs[end].pitch) * imgs[end].height, ++end;
+      while (end < n && (end == f || (sum < kPartBytes && bands_of(end) == 1))) sum += bytes_of(end), ++end;
       for (size_t i = f; i < end; ++i) upload(i, 0, imgs[i].height);
       after_uploads();
       if (status == DIBR_OK)
-        status = end - f == 1 && rows ? st->gpu->enqueue_rows(&imgs[f], &prms[f], &outs[f], 0, H)
+        status = end - f == 1 && own_rows(f) ? st->gpu->enqueue_rows(&imgs[f], &prms[f], &outs[f], 0, H)
                                       : st->gpu->enqueue_batch_device(static_cast<int>(end - f), &imgs[f], &prms[f],
                                                                       static_cast<int>(end - f), &outs[f]);
       after_launch();

@@ -68,3 +68,27 @@ def test_a_frame_alone(fake):
 def test_tuned_rows_per_unit_reach_a_frame_alone(fake, size):
     # (a batched launch, whose units have that many rows)
     assert _batch(fake, [size], rows_per_unit=16) == (_rows(size, 1), ["batch_kernel"])
+
+
+@pytest.mark.parametrize("sizes", [[HD, K4], [K4, HD], [HD, HD, HD, K4], [FHD, K4, HD, K4]])
+def test_large_frames_go_by_themselves(fake, sizes):
+    ups, kernels = _batch(fake, sizes)
+    assert ups == [r for s in sizes for r in _rows(s, 4 if s == K4 else 1)]
+    # between the large frames, the others: alone in a launch of their own, or (two 720p frames
+    # fill a part) together in a batched one
+    expect, k = [], 0
+    while k < len(sizes):
+        if sizes[k] == K4:
+            expect += ["band_kernel"] * 4
+            k += 1
+        elif sizes[k:k + 2] == [HD, HD]:
+            expect.append("batch_kernel")
+            k += 2
+        else:
+            expect.append("band_kernel")
+            k += 1
+    assert kernels == expect
+
+
+def test_cross_bilateral_frames_go_whole(fake):
+    assert _batch(fake, [HD, K4], depth_rule=D.DIBR_DEPTH_LUMA_XBF)[0] == _rows(HD, 1) + _rows(K4, 1)
