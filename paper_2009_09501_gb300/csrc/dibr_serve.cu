@@ -115,6 +115,19 @@ static void free_stream(ServeState *st, Stream &s) {
   st->resident -= s.bytes;
 }
 
+// A launch of a frame's own rows, alone in its part: not with the cross-bilateral depth, whose pass
+// takes the whole frame, nor where the tuning sets the rows of a batched launch's units.
+static bool own_rows(const dibr_params &p, const dibr_tuning &t) {
+  return p.depth_rule != DIBR_DEPTH_LUMA_XBF && t.rows_per_unit == 0;
+}
+
+// The row bands a frame is worth by its size (a large frame: more than one).
+static int row_bands(const dibr_params &p, const dibr_tuning &t, int64_t in_pitch, int H) {
+  if (!own_rows(p, t)) return 1;
+  const size_t parts = static_cast<size_t>(in_pitch) * H / kPartBytes;
+  return std::max(1, std::min(static_cast<int>(std::min(kMaxParts, parts)), H / 8));
+}
+
 // Scheduler: forms and enqueues batches.
 static void scheduler_loop(ServeState *st) {
   cudaSetDevice(st->gpu->device);
@@ -124,7 +137,7 @@ static void scheduler_loop(ServeState *st) {
   std::vector<dibr_outputs> outs;
   while (true) {
     InFlight b;
-    int others = 0;  // frames of earlier batches still in flight
+    int large = 0;  // large frames on their way: this batch's and those of earlier ones
     {
       std::unique_lock<std::mutex> lk(st->mu);
       auto ready = [&] {
@@ -162,8 +175,10 @@ static void scheduler_loop(ServeState *st) {
           more = true;
         }
       }
-      for (const auto &kv : st->streams) others += kv.second->in_flight;
-      others -= static_cast<int>(b.frames.size());
+      for (const auto &kv : st->streams) {
+        const Stream &s = *kv.second;
+        if (row_bands(s.p, st->gpu->tuning, s.in_pitch, s.H) > 1) large += s.in_flight;
+      }
       // descriptors of the batch (stream objects stay alive while they have frames in flight)
       imgs.clear();
       prms.clear();
@@ -232,20 +247,16 @@ static void scheduler_loop(ServeState *st) {
     // The batch goes through the three streams in parts, so that one part's download runs beside
     // the next one's upload (the host link bounds a batch; with the whole batch as one part, two
     // 1080p and two 4K frames took 906 us, 547 in parts): small frames together, a launch for each
-    // part of at least kPartBytes of input, and a large frame by itself in row bands.  With two
-    // frames or more in flight their copies fill the link already, and bands only add copies (4K
-    // frames streamed three at a time: 2,266 frames/s in bands, 2,370 whole).
+    // part of at least kPartBytes of input, and a large frame by itself, in row bands while at most
+    // two such frames are on their way.  (The copies of three or more fill the link without, and
+    // bands only add copies: a batch of four 4K frames 812 us in bands, 794 whole, of eight 1,480 and
+    // 1,435, streamed three at a time 2,266 and 2,370 frames/s; of two 437 and 439, and two 1080p
+    // and two 4K frames 531 and 547.)
     const size_t n = imgs.size();
-    // a launch of the frame's own rows: not with the cross-bilateral depth, whose pass takes the whole
-    // frame, nor where the tuning sets the rows of a batched launch's units
-    auto own_rows = [&](size_t f) { return prms[f].depth_rule != DIBR_DEPTH_LUMA_XBF && st->gpu->tuning.rows_per_unit == 0; };
-    auto bytes_of = [&](size_t f) { return static_cast<size_t>(imgs[f].pitch) * imgs[f].height; };
-    auto bands_of = [&](size_t f) {  // (of a large frame: more than one)
-      if (!own_rows(f)) return 1;
-      return std::max(1, std::min(static_cast<int>(std::min<size_t>(kMaxParts, bytes_of(f) / kPartBytes)), imgs[f].height / 8));
-    };
+    const dibr_tuning &tune = st->gpu->tuning;
+    auto bands_of = [&](size_t f) { return row_bands(prms[f], tune, imgs[f].pitch, imgs[f].height); };
     for (size_t f = 0; f < n && status == DIBR_OK;) {
-      const int H = imgs[f].height, bands = others < 2 ? bands_of(f) : 1;
+      const int H = imgs[f].height, bands = large <= 2 ? bands_of(f) : 1;
       if (bands > 1) {
         auto row = [&](int j) { return static_cast<int>(static_cast<int64_t>(j) * H / bands); };
         upload(f, 0, row(1));
@@ -261,11 +272,11 @@ static void scheduler_loop(ServeState *st) {
         continue;
       }
       size_t end = f, sum = 0;
-      while (end < n && (end == f || (sum < kPartBytes && bands_of(end) == 1))) sum += bytes_of(end), ++end;
+      while (end < n && (end == f || (sum < kPartBytes && bands_of(end) == 1))) sum += static_cast<size_t>(imgs[end].pitch) * imgs[end].height, ++end;
       for (size_t i = f; i < end; ++i) upload(i, 0, imgs[i].height);
       after_uploads();
       if (status == DIBR_OK)
-        status = end - f == 1 && own_rows(f) ? st->gpu->enqueue_rows(&imgs[f], &prms[f], &outs[f], 0, H)
+        status = end - f == 1 && own_rows(prms[f], tune) ? st->gpu->enqueue_rows(&imgs[f], &prms[f], &outs[f], 0, H)
                                       : st->gpu->enqueue_batch_device(static_cast<int>(end - f), &imgs[f], &prms[f],
                                                                       static_cast<int>(end - f), &outs[f]);
       after_launch();

@@ -92,3 +92,10 @@ def test_large_frames_go_by_themselves(fake, sizes):
 
 def test_cross_bilateral_frames_go_whole(fake):
     assert _batch(fake, [HD, K4], depth_rule=D.DIBR_DEPTH_LUMA_XBF)[0] == _rows(HD, 1) + _rows(K4, 1)
+
+
+@pytest.mark.parametrize("large,bands", [(1, 4), (2, 4), (3, 1), (8, 1)])
+def test_more_than_two_large_frames_go_whole(fake, large, bands):
+    ups, kernels = _batch(fake, [K4] * large + [FHD])
+    assert ups == _rows(K4, bands) * large + _rows(FHD, 1)
+    assert kernels == ["band_kernel"] * (bands * large + 1)
