@@ -131,7 +131,9 @@ typedef struct {
 /* Where the outputs go.  Pointers for outputs not requested in dibr_params.outputs are
  * ignored and may be NULL; requested ones must be non-NULL.  RGB outputs are width x
  * height x 3 with row pitch `pitch` (>= 3*width); the depth and holes outputs are width x
- * height with row pitch `depth_pitch` (>= width).  on_device as in dibr_image. */
+ * height with row pitch `depth_pitch` (>= width).  An output may lie over the input of its
+ * own image (which is then copied first, not in dibr_synthesize_batch_static).  on_device
+ * as in dibr_image. */
 typedef struct {
     uint8_t *anaglyph, *left, *right, *hsbs, *depth, *holes;
     int64_t pitch;

@@ -320,7 +320,7 @@ dibr_status dibr_ctx::encode_input(BandArgs &a, const uint8_t *dev_rgb, int64_t 
 dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p, const dibr_outputs *o) {
   const int W = img->width, H = img->height;
   const uint8_t *in = img->rgb;
-  const int64_t pitch = img->pitch;
+  int64_t pitch = img->pitch;
   // this launch may overlap the previous one (see below) only if that was the last work
   // on a stream the context owns, and neither is only recorded by a capture: a recorded launch
   // runs some other time, behind work this context does not know
@@ -341,16 +341,25 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   };
   auto meets = [](const Span &x, const Span &y) { return x.lo < y.hi && y.lo < x.hi; };
   bool scratch = false;  // context buffers written before the band kernel
+  dibr_status s;
+  // an output over the input: rows are read after others were written, so the input is copied first
+  if (in_place(*img, p->outputs, *o)) {
+    scratch = true;
+    const int64_t ap = round_up(3 * W, 16);
+    if ((s = ensure(input_copy, static_cast<size_t>(ap) * H)) != DIBR_OK) return s;
+    e = cudaMemcpy2DAsync(input_copy.ptr, ap, in, pitch, 3 * static_cast<size_t>(W), H, cudaMemcpyDeviceToDevice, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "copying an input under an output");
+    in = input_copy.ptr;
+    pitch = ap;
+  }
   int depth_src = p->depth_rule == DIBR_DEPTH_LUMA_BINOM5 ? DS_BINOM5
                   : p->depth_rule == DIBR_DEPTH_LUMA     ? DS_LUMA
                                                          : DS_GLOBAL;
   BandArgs &a = args;
   int smem = 0, per_sm = 1;
   const int zguard = band_tables(p);
-  dibr_status s;
   Span cur_depth;  // the cross-bilateral depth this frame's band launch reads
   if (depth_src == DS_GLOBAL) {
-    scratch = true;  // the band launch waits for the cross-bilateral one
     // two halves used by alternate frames, so that this frame's cross-bilateral launch may
     // start beside the previous frame's band launch: it reads this frame's input and writes
     // a half that launch does not read, when neither meets that launch's outputs
@@ -361,7 +370,8 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
     xbf_half ^= 1;
     cur_depth = span(dd, dp, H, W);
     const Span xin = span(in, pitch, H, 3 * static_cast<int64_t>(W));
-    bool after = may_overlap;
+    bool after = may_overlap && !scratch;
+    scratch = true;  // the band launch waits for the cross-bilateral one
     for (int k = 0; k < n_flights; ++k) {
       const Flight &f = flights[k];
       if (meets(cur_depth, f.in) || meets(cur_depth, f.depth)) after = false;
@@ -426,17 +436,16 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   // that one writes.)
   Span cur_in = span(in, pitch, H, 3 * static_cast<int64_t>(W)), cur_out[O_COUNT];
   int n_out = 0;
-  bool disjoint = may_overlap && !scratch, in_place = false;
+  bool disjoint = may_overlap && !scratch;
   for (int i = 0; i < O_COUNT; ++i) {
     if (!(a.outputs & kOutBits[i]) || !a.out[i]) continue;
-    cur_out[n_out] = span(a.out[i], is_map_output(i) ? a.depth_pitch : a.out_pitch, H,
+    cur_out[n_out++] = span(a.out[i], is_map_output(i) ? a.depth_pitch : a.out_pitch, H,
                           is_map_output(i) ? static_cast<int64_t>(W) : 3 * static_cast<int64_t>(W));
-    if (meets(cur_in, cur_out[n_out++])) in_place = true;
   }
   int again = -1;
   for (int k = 0; k < n_flights && disjoint; ++k) {
     const Flight &f = flights[k];
-    if (f.frame && !inpaint && !in_place && std::memcmp(&f.img, img, sizeof(*img)) == 0 &&
+    if (f.frame && !inpaint && std::memcmp(&f.img, img, sizeof(*img)) == 0 &&
         std::memcmp(&f.p, p, sizeof(*p)) == 0 && std::memcmp(&f.o, o, sizeof(*o)) == 0) {
       again = k;
       continue;
@@ -917,7 +926,7 @@ dibr_status dibr_ctx::synthesize_staged(const dibr_image *img, const dibr_params
 
 void dibr_ctx::release_buffers() {
   release_band_pipeline();
-  for (DevBuf *b : {&stage_in, &stage_out, &xbf_depth, &inpaint_scratch, &inpaint_order}) {
+  for (DevBuf *b : {&stage_in, &stage_out, &input_copy, &xbf_depth, &inpaint_scratch, &inpaint_order}) {
     dev_free(b->ptr);
     b->ptr = nullptr;
     b->bytes = 0;

@@ -48,7 +48,7 @@ static BatchShape shape_of(const dibr_image &im, const dibr_params &p, const dib
 }
 
 void dibr_ctx::release_batch_buffers() {
-  for (DevBuf *b : {&batch_desc, &batch_depth}) {
+  for (DevBuf *b : {&batch_desc, &batch_img, &batch_depth}) {
     dev_free(b->ptr);
     b->ptr = nullptr;
     b->bytes = 0;
@@ -131,12 +131,33 @@ dibr_status dibr_ctx::enqueue_grouped(int n, const dibr_image *imgs, const dibr_
                                       const dibr_outputs *outs) {
   prev_band = false;
   if (n == 0) return DIBR_OK;
+  dibr_status s;
+  // --- inputs under an output of their own image are copied first (as for one frame)
+  size_t copy_bytes = 0;
+  for (int i = 0; i < n; ++i)
+    if (in_place(imgs[i], p[n_params == 1 ? 0 : i].outputs, outs[i])) copy_bytes += static_cast<size_t>(round_up(3 * imgs[i].width, 16)) * imgs[i].height;
+  std::vector<dibr_image> moved;
+  if (copy_bytes) {
+    if ((s = ensure(batch_img, copy_bytes)) != DIBR_OK) return s;
+    moved.assign(imgs, imgs + n);
+    uint8_t *to = batch_img.ptr;
+    for (int i = 0; i < n; ++i) {
+      dibr_image &im = moved[i];
+      if (!in_place(im, p[n_params == 1 ? 0 : i].outputs, outs[i])) continue;
+      const int64_t ap = round_up(3 * im.width, 16);
+      const cudaError_t e = cudaMemcpy2DAsync(to, ap, im.rgb, im.pitch, 3 * static_cast<size_t>(im.width), im.height, cudaMemcpyDeviceToDevice, stream);
+      if (e != cudaSuccess) return cuda_fail(e, "copying an input under an output");
+      im.rgb = to;
+      im.pitch = ap;
+      to += static_cast<size_t>(ap) * im.height;
+    }
+    imgs = moved.data();
+  }
   // --- cross-bilateral depths first, into one buffer
   size_t depth_bytes = 0;
   for (int i = 0; i < n; ++i)
     if (p[n_params == 1 ? 0 : i].depth_rule == DIBR_DEPTH_LUMA_XBF)
       depth_bytes += static_cast<size_t>(round_up(imgs[i].width, 16)) * imgs[i].height;
-  dibr_status s;
   if (depth_bytes && (s = ensure(batch_depth, depth_bytes)) != DIBR_OK) return s;
   size_t dof = 0;
   std::vector<const uint8_t *> depth_in(n, nullptr);

@@ -56,7 +56,7 @@ struct dibr_ctx {
   std::mutex err_mu;
   std::string last_error, last_error_copy;
 
-  dibr::DevBuf stage_in, stage_out, xbf_depth, inpaint_scratch, inpaint_order;
+  dibr::DevBuf stage_in, stage_out, input_copy, xbf_depth, inpaint_scratch, inpaint_order;
   dibr::BandArgs args;  // scratch for one launch (large: keeps it off the stack)
   // the shift tables in args (and their guard width) were built for these disparity
   // parameters {rule, P, T}; rebuilt only when a call brings others

@@ -221,6 +221,24 @@ inline bool rows_aligned(const uint8_t *p, int64_t pitch) {
   return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (pitch & 15) == 0;
 }
 
+// Whether an output lies over the input's bytes (H rows each; rows of wa bytes pa apart from a, of
+// wb bytes pb apart from b).  Two windows of one buffer with one pitch may lie side by side.
+inline bool rows_meet(const uint8_t *a, int64_t pa, int64_t wa, const uint8_t *b, int64_t pb, int64_t wb, int H) {
+  const int64_t a0 = static_cast<int64_t>(reinterpret_cast<uintptr_t>(a)), b0 = static_cast<int64_t>(reinterpret_cast<uintptr_t>(b));
+  if (a0 + (H - 1) * pa + wa <= b0 || b0 + (H - 1) * pb + wb <= a0) return false;
+  if (pa != pb) return true;
+  const int64_t d = ((b0 - a0) % pa + pa) % pa;  // from a row of a to the next one of b
+  return d < wa || d + wb > pa;
+}
+inline bool in_place(const dibr_image &img, uint32_t outputs, const dibr_outputs &o) {
+  for (int i = 0; i < O_COUNT; ++i)
+    if ((outputs & kOutBits[i]) &&
+        rows_meet(img.rgb, img.pitch, 3 * static_cast<int64_t>(img.width), out_slot(o, i), is_map_output(i) ? o.depth_pitch : o.pitch,
+                  (is_map_output(i) ? 1 : 3) * static_cast<int64_t>(img.width), img.height))
+      return true;
+  return false;
+}
+
 inline int chunks_of(int width) { return (width + kChunk - 1) / kChunk; }
 // Chunks of a z-buffer row: shifted by up to 15 columns in the modes that shift.
 inline int zchunks_of(int width, int out_mode) {
