@@ -74,15 +74,6 @@ void dibr_ctx::release_batch_buffers() {
 // frames 172 us, 70 so -- the shared launch's descriptors take an upload.)
 constexpr int kOwnLaunchRows = 4;
 
-// CTAs per SM of the two-row plan; 0: does not fit.
-static int two_row_ctas(const BatchShape &s, const BatchLimits &lim) {
-  const int nc = block_of(s), min_nb = 4;
-  const int tot = band_smem_layout(min_nb, slot_bytes(s.width, s.aligned), chunks_of(s.width), s.nchz, nc / 32, lim.zguard, 2).total;
-  if (tot > lim.band.max_smem) return 0;
-  const int per = std::min(lim.band.smem_per_sm / (tot + 1024), std::min(65536 / (nc * 128), 2048 / nc));
-  return lim.band.ctas_per_sm > 0 ? std::min(per, lim.band.ctas_per_sm) : per;
-}
-
 dibr_status dibr_ctx::enqueue_batch_device(int n, const dibr_image *imgs, const dibr_params *p, int n_params,
                                            const dibr_outputs *outs) {
   if (n == 0) return DIBR_OK;
@@ -93,7 +84,8 @@ dibr_status dibr_ctx::enqueue_batch_device(int n, const dibr_image *imgs, const 
     int cl = 0;
     BatchClass c[1];
     const bool fits = plan_batch_classes(1, &shape, lim, &cl, c) == 1;
-    const int two = fits ? two_row_ctas(shape, lim) : 0;
+    const int two = plan_rows(2, lim.band, block_of(shape), slot_bytes(shape.width, shape.aligned), chunks_of(shape.width), shape.nchz,
+                              lim.zguard, 4).per;
     const int64_t slots = static_cast<int64_t>(num_sms) * (two ? two : fits ? c[0].per : 1);
     bool big = fits && tuning.rows_per_unit == 0 && imgs[i].height >= kOwnLaunchRows * slots;
     const auto t = class_tune.find(block_of(shape));

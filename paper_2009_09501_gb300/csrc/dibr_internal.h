@@ -272,28 +272,32 @@ struct BandLimits {
   int ring_slots, ctas_per_sm;
 };
 
-// The most CTAs per SM within the limits (128 registers per thread: the kernels' launch bound;
-// 2048 threads per SM), two z-buffer rows per view unless one leaves room for more CTAs (rows of
-// 3857 to 4096 pixels: two CTAs instead of one, a 4031 x 3023
-// frame 99 -> 66 us; 1080p: four instead of three, 10.3 -> 9.1), and the deepest ring.  Returns
-// false if no plan fits.
-inline bool plan_smem(BandPlan &p, const BandLimits &lim, int nc, int srow, int nch, int nchz, int zguard, int min_nb) {
+// The plan with zp z-buffer rows per view: the most CTAs per SM within the limits (128 registers per
+// thread: the kernels' launch bound; 2048 threads per SM) and the deepest ring with that many.
+// per = 0: none fits.
+inline BandPlan plan_rows(int zp, const BandLimits &lim, int nc, int srow, int nch, int nchz, int zguard, int min_nb) {
   const int max_nb = lim.ring_slots <= 0 ? kMaxRing : lim.ring_slots < min_nb ? min_nb : lim.ring_slots < kMaxRing ? lim.ring_slots : kMaxRing;
   const int by_regs = 65536 / (nc * 128), by_threads = 2048 / nc;
-  p = BandPlan{0, 0, 0, 0};
-  for (int zp = 2; zp >= 1; --zp) {
-    BandPlan q{0, zp, 0, 0};
-    for (int nb = min_nb; nb <= max_nb; ++nb) {
-      const int tot = band_smem_layout(nb, srow, nch, nchz, nc / 32, zguard, zp).total;
-      if (tot > lim.max_smem) continue;
-      int per = lim.smem_per_sm / (tot + 1024);
-      if (per > by_regs) per = by_regs;
-      if (per > by_threads) per = by_threads;
-      if (lim.ctas_per_sm > 0 && per > lim.ctas_per_sm) per = lim.ctas_per_sm;
-      if (per >= 1 && per >= q.per) q = BandPlan{nb, zp, per, tot};
-    }
-    if (q.per > p.per) p = q;
+  BandPlan q{0, zp, 0, 0};
+  for (int nb = min_nb; nb <= max_nb; ++nb) {
+    const int tot = band_smem_layout(nb, srow, nch, nchz, nc / 32, zguard, zp).total;
+    if (tot > lim.max_smem) continue;
+    int per = lim.smem_per_sm / (tot + 1024);
+    if (per > by_regs) per = by_regs;
+    if (per > by_threads) per = by_threads;
+    if (lim.ctas_per_sm > 0 && per > lim.ctas_per_sm) per = lim.ctas_per_sm;
+    if (per >= 1 && per >= q.per) q = BandPlan{nb, zp, per, tot};
   }
+  return q;
+}
+
+// Two z-buffer rows per view unless one leaves room for more CTAs on the SM (rows of 3857 to 4096
+// pixels: two CTAs instead of one, a 4031 x 3023 frame 99 -> 66 us; 1080p: four instead of three,
+// 10.3 -> 9.1).  Returns false if no plan fits.
+inline bool plan_smem(BandPlan &p, const BandLimits &lim, int nc, int srow, int nch, int nchz, int zguard, int min_nb) {
+  p = plan_rows(2, lim, nc, srow, nch, nchz, zguard, min_nb);
+  const BandPlan one = plan_rows(1, lim, nc, srow, nch, nchz, zguard, min_nb);
+  if (one.per > p.per) p = one;
   return p.per >= 1;
 }
 

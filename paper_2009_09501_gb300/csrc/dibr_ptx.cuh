@@ -54,10 +54,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// Waits for the phase of `parity` to complete; gives up after limit_ns nanoseconds and
-// returns false (the caller records the failure and unwinds without touching the GPU's
-// state further).
-__device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity) {
+// Non-blocking test of the completion of the phase of `parity`.
+__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
@@ -73,9 +71,12 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity) {
 // unit, or -- for limits below that -- a test that does not block, so that such a limit
 // takes effect.
 __device__ __forceinline__ bool mbar_attempt(uint64_t *bar, uint32_t parity, unsigned long long limit_ns) {
-  return limit_ns < 500000ull ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity);
+  return limit_ns < 500000ull ? mbar_test(bar, parity) : mbar_try_wait(bar, parity);
 }
 
+// Waits for the phase of `parity` to complete; gives up after limit_ns nanoseconds and
+// returns false (the caller records the failure and unwinds without touching the GPU's
+// state further).
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity,
                                                   unsigned long long limit_ns) {
   if (mbar_attempt(bar, parity, limit_ns)) return true;
@@ -163,17 +164,11 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
 __device__ __forceinline__ void lds_u32_if(uint32_t &v, uint32_t a, bool pred) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.shared.u32 %0, [%1];\n\t}" : "+r"(v) : "r"(a), "r"(static_cast<uint32_t>(pred)));
 }
-__device__ __forceinline__ int4 lds_s32x4(uint32_t a) {
-  int4 v;
-  asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-  return v;
-}
 __device__ __forceinline__ uint4 lds_u32x4(uint32_t a) {
   uint4 v;
   asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
   return v;
 }
-// atomic minimum without a returned value
 // Bytes at a, a+32, a+64, a+96: one lane's depths for four consecutive 32-column steps.
 __device__ __forceinline__ void lds_u8_step32x4(uint32_t a, uint32_t (&v)[4]) {
   asm volatile(
@@ -199,15 +194,6 @@ __device__ __forceinline__ void lds_u32_pair_step96x4(uint32_t a, uint32_t (&v)[
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
       : "r"(a));
 }
-__device__ __forceinline__ void reds_min(uint32_t a, uint32_t v) {
-  asm volatile("red.shared.min.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-
-__device__ __forceinline__ uint2 lds_u32x2(uint32_t a) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
-  return v;
-}
 __device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) {
   asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
@@ -232,28 +218,10 @@ __device__ __forceinline__ uint32_t lanemask_gt() {
   return m;
 }
 
-// Non-blocking test of the completion of the phase of `parity`.
-__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
 // Programmatic dependent launch: let the next launch on the stream start / wait for the
 // previous one (with its memory) to complete; both are no-ops for a launch without it.
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// Named barrier 1 over the consumer threads only.
-__device__ __forceinline__ void consumer_sync(int nthreads) {
-  asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
-}
 
 // Named barrier 1 with an OR over the participating threads' predicates; every thread
 // gets the same result, so a failure seen by one thread unwinds all of them together.
