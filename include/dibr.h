@@ -185,7 +185,9 @@ const char *dibr_last_error(dibr_ctx *ctx);
  * (dibr_config.cuda_stream NULL), the caller may record events on it and wait for it but
  * enqueues no work of its own there; consecutive dibr_enqueue_image calls whose buffers
  * are disjoint then overlap: the next frame starts in the SMs the previous one has left
- * (a frame still completes only after the one before it). */
+ * (a frame still completes only after the one before it).  Frames enqueued while the
+ * stream is being captured are recorded one after the other, once the context's buffers
+ * have been allocated by a frame of that kind. */
 void *dibr_stream(dibr_ctx *ctx);
 
 /* One frame, blocking: returns when the outputs are written (host or device).  Host
@@ -215,14 +217,14 @@ dibr_status dibr_enqueue_batch(dibr_ctx *ctx, int n, const dibr_image *imgs,
 
 /* Autotuner of the batched launches (the paper has no counterpart; it changes speed,
  * never results).  The images are grouped by size class -- the block width of their rows,
- * one thread per 16 columns rounded up to whole warps -- and each class is run alone
+ * one thread per 16 columns (of up to 15 more where output rows do not start on 16-byte
+ * boundaries) rounded up to whole warps -- and each class is run alone
  * (reps timed repetitions after one warm-up, CUDA events on the context's stream) under
  * every candidate plan: a band launch of its own per image, or the shared persistent
  * launch with rows per work unit in {automatic, 2, 4, 8, 16, 32, 64}, CTAs per SM
  * {automatic, 1} and ring slots {automatic, 4}.  The fastest plan of each class is kept in
- * the context and used by every later dibr_synthesize_batch / dibr_enqueue_batch (and
- * serving batch) whose images fall in that class, where the matching dibr_set_tuning
- * knob is automatic.  All buffers must be device memory; the outputs are written (with
+ * the context and used by every later dibr_synthesize_batch / dibr_enqueue_batch whose
+ * images fall in that class, where the matching dibr_set_tuning knob is automatic.  All buffers must be device memory; the outputs are written (with
  * the final results) by the timed runs.  Blocking. */
 dibr_status dibr_autotune_batch(dibr_ctx *ctx, int n, const dibr_image *imgs, const dibr_params *p,
                                 int n_params, const dibr_outputs *outs, int reps);
@@ -245,7 +247,7 @@ dibr_status dibr_tuning_load(dibr_ctx *ctx, const char *path);
  * data, which every GPU that loads the library holds until the process exits.
  *   - Inputs and outputs: device memory of the current device, as for dibr_enqueue_batch.
  *     Input rows must be whole 16-byte units: 16-byte aligned base and pitch, 3*width a
- *     multiple of 16 (other images would need a repacking buffer).
+ *     multiple of 16.
  *   - Limits: 1..64 images; depth rules DIBR_DEPTH_LUMA and DIBR_DEPTH_LUMA_BINOM5 only
  *     (the cross-bilateral rule needs a depth buffer); at most 8192 work units (rows per
  *     unit grow to fit).  Anything beyond returns DIBR_E_INVALID, with no error text.
@@ -273,17 +275,21 @@ dibr_status dibr_synthesize_batch_static(int n, const dibr_image *imgs, const di
  *   l2_prefetch    1: each CTA prefetches its later input rows into L2 at launch;
  *                  2: it does not;
  *   rows_per_unit  rows per work unit of a batched launch (dibr_synthesize_batch and
- *                  the serving loop); automatic: one unit per SM slot when an image group
- *                  is small (one 4K frame: 8 rows), 32 rows otherwise;
+ *                  the serving loop, whose frames then all take such launches);
+ *                  automatic: one unit per SM slot when an image group is small (one 4K
+ *                  frame: 8 rows), 32 rows otherwise;
  *   host_bands     row bands of dibr_synthesize_image with host input and outputs (the
  *                  bands' uploads, kernels and downloads overlap), 1..8; automatic: 4 from
  *                  4 MB of input, else 1;
  *   frames_in_flight  1..16: when a frame is enqueued on the context's own stream while
- *                  earlier work is still queued there, and it shares no buffer with the
- *                  frame before it, its launch takes 1/n of the SM slots (in taller row
- *                  bands), so that n consecutive frames run side by side; 1: every launch
- *                  spreads over all SMs.  A launch on an idle stream always does.
- *                  Automatic: 7.
+ *                  earlier work is still queued there, and no buffer that it or a frame that
+ *                  may still run writes is one of the other's, its launch takes 1/n of the
+ *                  SM slots (in taller row bands), so that n consecutive frames run side by
+ *                  side (a repeat of a frame that may still run, with the same records, may
+ *                  run beside it: both write the same bytes); 1: every launch spreads over
+ *                  all SMs.  A launch on an idle stream, one behind a frame whose buffers it
+ *                  shares, and every frame with DIBR_FILL_INPAINT2D, whose launches nothing
+ *                  runs beside, always do.  Automatic: 7.
  * dibr_set_tuning() rejects out-of-range values with DIBR_E_INVALID. */
 typedef struct {
     int32_t ring_slots, ctas_per_sm, load_mode, l2_prefetch, rows_per_unit, host_bands;
@@ -306,9 +312,11 @@ dibr_status dibr_set_wait_limit(dibr_ctx *ctx, uint64_t limit_ns);
 
 /* ------------------------------------------------------------------ serving loop ---
  * Concurrent video streams with continuous batching: frames submitted on any open
- * stream are gathered by a scheduler thread, copied to per-stream device buffers on a
- * copy stream, synthesized together in one batched launch, and copied back on a second
- * copy stream; completions are returned by dibr_poll(). */
+ * stream are gathered by a scheduler thread into batches.  A batch goes in parts -- small
+ * frames together, a large one by itself or in row bands -- that are copied to per-stream
+ * device buffers on a copy stream, synthesized, and copied back on a second copy stream,
+ * so that one part's copies run beside another's; completions are returned by
+ * dibr_poll() when the whole batch is back. */
 typedef struct {
     int32_t stream_id;
     int32_t status;           /* dibr_status of this frame */

@@ -433,7 +433,8 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   // Overlap with the band launches before it on the stream when neither reads or writes what
   // the other writes: this launch then starts in the SMs the previous one leaves and only
   // its exit waits for it.  (The same frame again, a repeat of one in flight, writes the bytes
-  // that one writes.)
+  // that one writes: whatever changes what it reads or uses what it writes in between is a launch
+  // of this context, which starts the list anew, or waits for that one to complete.)
   Span cur_in = span(in, pitch, H, 3 * static_cast<int64_t>(W)), cur_out[O_COUNT];
   int n_out = 0;
   bool disjoint = may_overlap && !scratch;
@@ -466,9 +467,9 @@ dibr_status dibr_ctx::enqueue_device(const dibr_image *img, const dibr_params *p
   // one after the other across every SM.  Both CTAs of an SM must fit at once.  Not with the
   // 2-D fill: its launches follow this one and nothing of another frame runs beside it, so a
   // share of the SMs only made it longer (4K frames back to back 334 us, 114 on every SM).
-  // Two CTAs an SM are enough there, unless the tuning says how many: more leave a CTA two rows beside the five its first row
-  // needs, and the launches behind it no room to be ready in (1080p 71 us with four, 49 with
-  // two and with one; 1440p 91, 65 and 75).
+  // Two CTAs an SM are enough there, unless the tuning says how many: more leave a CTA two rows
+  // beside the five its first row needs, and the launches behind it no room to be ready in (1080p
+  // 71 us with four, 49 with two and with one; 1440p 91, 65 and 75).
   const int fif = tuning.frames_in_flight > 0 ? tuning.frames_in_flight : kFramesInFlight;
   const int full_grid = a.grid;
   if (disjoint && !inpaint && fif > 1 && per_sm >= 2 && driver().query(stream) == CUDA_ERROR_NOT_READY)

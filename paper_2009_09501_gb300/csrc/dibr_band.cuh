@@ -25,15 +25,15 @@
 //   C  reads its 16 targets' entries, fills holes (register sweeps; the entries carried
 //      across chunks come from the neighbouring lanes by shuffle, across warps from a
 //      per-warp summary in shared memory), formats and stores the outputs, and clears
-//      its warp's targets for the row two rows later.
-// Rows interleave as A(y+1), B(y+1), C(y).  There is no CTA-wide barrier per row: C of a
-// row waits on an mbarrier every warp arrives on after B of that row (a row earlier), B of
-// a row waits on one every warp arrives on once it has published its summary of the row
-// two rows before and cleared its targets there (the same z-buffer), and a warp that needs
-// an entry from outside its own targets waits on that second one for its own row.  The
-// barriers come in pairs used by alternate rows.  Every wait is bounded (%globaltimer); a
-// wait that gives up sets a bit of the status word and the CTA unwinds after letting its
-// own copies land.
+//      its warp's targets for the next row that uses the same z-buffer.
+// With two z-buffer rows per view (used by alternate rows) rows interleave as A(y+1), B(y+1),
+// C(y); with one they run A(y), B(y), C(y).  There is no CTA-wide barrier per row: C of a row
+// waits on an mbarrier every warp arrives on after B of that row, B of a row waits on one every
+// warp arrives on once it has published its summary of the row before that used the z-buffer
+// (two rows back, or one) and cleared its targets there, and a warp that needs an entry from
+// outside its own targets waits on that second one for its own row.  The barriers come in pairs
+// used by alternate rows.  Every wait is bounded (%globaltimer); a wait that gives up sets a bit
+// of the status word and the CTA unwinds after letting its own copies land.
 //
 // Rows may start anywhere (tight rows of a width that is no multiple of 16, an offset base): a
 // ring slot then holds the 16-byte units a row touches, its first byte at `lead`; the luminance
@@ -41,8 +41,9 @@
 // z-buffer keeps target x at x + shift, with the row's shift (0..15) chosen so that every thread's
 // 16 targets start on a 16-byte boundary of the output row; only the two chunks cut by the row's
 // ends are stored by words and bytes.  That is the RAG template flag: a 4031 x 3023 photo with
-// tight rows 780 -> 61 us (of it 107 -> 66 by one z-buffer row per view), 1366 x 768 side by side 29.6 -> 8.9 us (repacked by a strided copy
-// and stored by bytes before); aligned images keep instances without it.
+// tight rows 780 -> 61 us (of it 107 -> 66 by one z-buffer row per view), 1366 x 768 side by side
+// 29.6 -> 8.9 us (repacked by a strided copy and stored by bytes before); aligned images keep
+// instances without it.
 //
 // Instances: the requested outputs are read from the arguments, or fixed at compile time for
 // the two sets the workloads use (left + right + anaglyph, anaglyph alone; binomial depth,
@@ -835,7 +836,7 @@ __device__ __forceinline__ bool run_band(const Job &a, const Shm &m, int ys, int
       // Fig. 3 literally: target x samples column trunc(x + s(d)) = x + floor(s(d)), but 0
       // when -1 < x + s(d) < 0; its own column when that lies outside the row.  From the row
       // in shared memory into the z-buffers, from which C formats it like a row of the forward
-      // warp without holes (1080p: 8.8 us with byte loads from global memory in C, 7.8 so).
+      // warp without holes (1080p: 8.9 us with byte loads from global memory in C, 6.5 so).
       const int ng = (warp_hi - warp_lo + 127) >> 7;  // groups of 4 x 32 columns holding some
 #pragma unroll 1
       for (int g = 0; g < ng; ++g) {

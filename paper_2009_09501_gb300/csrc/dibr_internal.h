@@ -180,7 +180,7 @@ struct BatchArgs {
 };
 
 // Output sets with kernel instances of their own (outputs fixed at compile time): binomial
-// depth, forward warp, whole-word stores.
+// depth, forward warp, rows stored by words (aligned ones, or ragged ones shifted alike: OM_SHIFT).
 constexpr uint32_t kSetStereo = DIBR_OUT_ANAGLYPH | DIBR_OUT_LEFT | DIBR_OUT_RIGHT;
 constexpr uint32_t kSetAnaglyph = DIBR_OUT_ANAGLYPH;
 

@@ -67,7 +67,7 @@ struct Stream {
 
 constexpr int kStatusRing = 1024;  // > streams x slots: one entry per batch in flight
 
-struct InFlight {  // one batched launch
+struct InFlight {  // one batch
   cudaEvent_t done;
   int status_slot;  // this batch's status word on the device and its pinned copy
   std::vector<std::pair<int, int>> frames;  // (stream id, slot)
@@ -197,7 +197,7 @@ static void scheduler_loop(ServeState *st) {
         outs.push_back(o);
       }
     }
-    // uploads (copy stream) -> batched launch (compute stream) -> downloads (copy stream)
+    // uploads (copy stream) -> launches (compute stream) -> downloads (copy stream), in parts
     dibr_status status = DIBR_OK;
     cudaEvent_t up = st->ev_up, comp = st->ev_comp;
     b.done = nullptr;

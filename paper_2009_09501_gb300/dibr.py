@@ -301,7 +301,8 @@ def outputs_struct(outs, pitch=None, depth_pitch=None):
 
 def block_threads(width):
     """The size class of an image in batched launches: threads per block for its rows (one
-    per 16 columns, rounded up to whole warps)."""
+    per 16 columns, rounded up to whole warps; outputs whose rows start off 16-byte boundaries
+    count up to 15 columns more)."""
     return ((width + 15) // 16 + 31) // 32 * 32
 
 
