@@ -17,7 +17,9 @@ class Fake:
         real = D.load()  # (builds the objects if they are missing or old)
         cuda = os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc())))
         so = os.path.join(str(folder), "libdibr_fake.so")
-        objs = [o for o in sorted(glob.glob(os.path.join(B.BUILD_DIR, "*.o"))) if os.path.exists(os.path.join(B.CSRC, os.path.basename(o)[:-1] + "cu"))]
+        objs = [os.path.join(B.BUILD_DIR, os.path.basename(c)[:-2] + "o") for c in sorted(glob.glob(os.path.join(B.CSRC, "*.cu")))]
+        if not all(os.path.exists(o) for o in objs):  # (the library without its objects)
+            B.build(force=True)
         cmd = ["g++", "-std=c++17", "-O1", "-w", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I" + B.INCLUDE, "-I" + B.CSRC,
                "-I" + os.path.join(cuda, "include"), os.path.join(HERE, "fake_cudart.cpp")] + objs + ["-lpthread", "-o", so]
         r = subprocess.run(cmd, capture_output=True, text=True)
