@@ -876,12 +876,12 @@ dibr_status dibr_ctx::synthesize_staged(const dibr_image *img, const dibr_params
   prev_band = false;  // copies precede the launch
   // row bands when both sides of the call are in host memory and every row band is
   // independent of the others' results (not with the 2-D fill or the cross-bilateral depth,
-  // which need the whole frame first)
+  // which need the whole frame first), nor written over another's input
   // (automatic: from 4 MB of input -- 1080p anaglyph 107 us in two bands, 102 in one, 95 in four, all
   // three outputs 179, 171 and 173; 720p 104, 98 and 104)
   const int bands = tuning.host_bands > 0 ? std::min(tuning.host_bands, H) : 3ll * W * H >= (4 << 20) ? std::min(4, H) : 1;
   if (bands > 1 && !img->on_device && !o->on_device && p->hole_fill == DIBR_FILL_ROW &&
-      p->depth_rule != DIBR_DEPTH_LUMA_XBF)
+      p->depth_rule != DIBR_DEPTH_LUMA_XBF && bands_in_order(*img, p->outputs, *o))
     return synthesize_banded(img, p, o, bands);
   dibr_image din = *img;
   dibr_outputs dout = *o;

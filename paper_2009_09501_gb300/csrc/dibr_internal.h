@@ -239,6 +239,19 @@ inline bool in_place(const dibr_image &img, uint32_t outputs, const dibr_outputs
   return false;
 }
 
+// Host buffers: whether row bands of the outputs may be written while later rows of the input are
+// still to be read, which they may unless an output's rows reach past the input's row of that number.
+inline bool bands_in_order(const dibr_image &img, uint32_t outputs, const dibr_outputs &o) {
+  const int64_t row = 3 * static_cast<int64_t>(img.width), first = static_cast<int64_t>(reinterpret_cast<uintptr_t>(img.rgb));
+  for (int i = 0; i < O_COUNT; ++i) {
+    if (!(outputs & kOutBits[i])) continue;
+    const int64_t pitch = is_map_output(i) ? o.depth_pitch : o.pitch, width = is_map_output(i) ? img.width : row;
+    if (pitch <= img.pitch && static_cast<int64_t>(reinterpret_cast<uintptr_t>(out_slot(o, i))) + width <= first + img.pitch) continue;
+    if (rows_meet(img.rgb, img.pitch, row, out_slot(o, i), pitch, width, img.height)) return false;
+  }
+  return true;
+}
+
 inline int chunks_of(int width) { return (width + kChunk - 1) / kChunk; }
 // Chunks of a z-buffer row: shifted by up to 15 columns in the modes that shift.
 inline int zchunks_of(int width, int out_mode) {

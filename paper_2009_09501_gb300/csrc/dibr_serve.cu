@@ -254,7 +254,9 @@ static void scheduler_loop(ServeState *st) {
     // and two 4K frames 531 and 547.)
     const size_t n = imgs.size();
     const dibr_tuning &tune = st->gpu->tuning;
-    auto bands_of = [&](size_t f) { return row_bands(prms[f], tune, imgs[f].pitch, imgs[f].height); };
+    auto bands_of = [&](size_t f) {
+      return bands_in_order(b.meta[f].in, prms[f].outputs, b.meta[f].out) ? row_bands(prms[f], tune, imgs[f].pitch, imgs[f].height) : 1;
+    };
     for (size_t f = 0; f < n && status == DIBR_OK;) {
       const int H = imgs[f].height, bands = large <= 2 ? bands_of(f) : 1;
       if (bands > 1) {
