@@ -442,18 +442,26 @@ template <class Whole, class Part>
 __host__ __device__ inline void frame_units(const uint8_t *view, int64_t pitch, int W, int H, int bx0, int by0, int bh,
                                             int lane, Whole whole, Part part) {
   const int64_t row_bytes = 3 * static_cast<int64_t>(W);
-  const uint8_t *const end = view + (H - 1) * pitch + row_bytes;
-  const int first = by0 > 0 ? by0 - 1 : 0, last = by0 + bh < H ? by0 + bh : H - 1;
-  const bool inside = first * pitch >= 15 && (H - 1 - last) * pitch >= 15;
+  const int last = by0 + bh < H ? by0 + bh : H - 1;
+  const bool inside = by0 > 5 && H - last > 5;  // five rows at least (15 bytes) before and behind the frame
   const int j0 = by0 == 0 && (lane >> 3) == 0 ? 4 : lane >> 3;  // (no row above the image)
-  const uint8_t *row = view + (by0 - 1 + j0) * pitch;
-  for (int j = j0; j <= last - by0 + 1; j += 4, row += 4 * pitch) {
-    const uintptr_t at = reinterpret_cast<uintptr_t>(row + 3 * static_cast<int64_t>(bx0 - 1)) & ~static_cast<uintptr_t>(15);
-    const uint8_t *const u = reinterpret_cast<const uint8_t *>(at) + 16 * (lane & 7);
-    if (u + 16 <= row || u >= row + row_bytes) continue;
-    if (inside || (u >= view && u + 16 <= end)) whole(j, u);
-    else part(j, u, u < view ? static_cast<int>(view - u) : 0, u + 16 > end ? static_cast<int>(end - u) : 16);
+  auto each = [&](auto visit) {
+    const uint8_t *row = view + (by0 - 1 + j0) * pitch;
+    for (int j = j0; j <= last - by0 + 1; j += 4, row += 4 * pitch) {
+      const uintptr_t at = reinterpret_cast<uintptr_t>(row + 3 * static_cast<int64_t>(bx0 - 1)) & ~static_cast<uintptr_t>(15);
+      const uint8_t *const u = reinterpret_cast<const uint8_t *>(at) + 16 * (lane & 7);
+      if (u + 16 > row && u < row + row_bytes) visit(j, u);
+    }
+  };
+  if (inside) {
+    each(whole);
+    return;
   }
+  each([&](int j, const uint8_t *u) {
+    const uint8_t *const end = view + (H - 1) * pitch + row_bytes;
+    if (u >= view && u + 16 <= end) whole(j, u);
+    else part(j, u, u < view ? static_cast<int>(view - u) : 0, u + 16 > end ? static_cast<int>(end - u) : 16);
+  });
 }
 
 // Host launchers (dibr_band*.cu, dibr_xbf.cu, dibr_inpaint.cu).
