@@ -285,9 +285,9 @@ dibr_status dibr_synthesize_batch_static(int n, const dibr_image *imgs, const di
  *                  earlier work is still queued there, and no buffer that it or a frame that
  *                  may still run writes is one of the other's, its launch takes 1/n of the
  *                  SM slots (in taller row bands), so that n consecutive frames run side by
- *                  side (a repeat of a frame that may still run, with the same records, may
- *                  run beside it: both write the same bytes); 1: every launch spreads over
- *                  all SMs.  A launch on an idle stream, one behind a frame whose buffers it
+ *                  side (a frame with the records of one that may still run, as in a ring of
+ *                  buffer sets, needs no wait for that one: while both run they read and
+ *                  write the same bytes); 1: every launch spreads over all SMs.  A launch on an idle stream, one behind a frame whose buffers it
  *                  shares, and every frame with DIBR_FILL_INPAINT2D, whose launches nothing
  *                  runs beside, always do.  Automatic: 7.
  * dibr_set_tuning() rejects out-of-range values with DIBR_E_INVALID. */
