@@ -24,7 +24,7 @@
 //
 // Bound by the integer pipe and issue while every SM has 32 warps, then by the latency of the
 // last items' steps.  A 4K frame with 8 % holes (11,732 items, 26 steps with visits each): the
-// kernel 71 us, 46 M warp instructions; the frame with its band launch 109-117 us.  When every
+// kernel 71 us, 46 M warp instructions; the frame with its band launch 108-118 us.  When every
 // dirty pixel was visited one at a time, the flags were read from the map and the colours
 // from the view by each item, byte by byte, and all parts of a block shared one origin: 125
 // us, 89 M, 170 us.
